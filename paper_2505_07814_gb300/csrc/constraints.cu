@@ -4,16 +4,13 @@
 //   probe orthogonalisation  k_gram (FP64 Gram-matrix partials of the probe modes), k_ortho_eig
 //                            (one warp: complex Jacobi eigensolver in FP64, modes sorted by power),
 //                            k_ortho_apply (each pixel's modes mixed by the eigenvectors, in place);
-//   k_z filter (Eq. 10-12)   the filter W_a is real and even in k, so one complex 3D DFT of
-//                            z = amp + i phase filters both real arrays: k_lines along x, then y
-//                            (forward), k_kz_columns (depth DFT, W_a / (Nz H W), inverse depth DFT
-//                            per (k_y, k_x) column), k_lines along y, then x (inverse); the last
-//                            pass writes amp and phase with the relaxation;
+//   k_z filter (Eq. 10-12)   kz_filter.cuh: k_kz_lines along x and y, k_kz_depth, k_kz_lines back;
 //   depth blur, positivity   k_constrain (Eq. 13 and the phase clip).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <string.h>
 
+#include "kz_filter.cuh"
 #include "pty_internal.h"
 
 namespace pty {
@@ -135,184 +132,6 @@ static int launch_constrain(float* amp, float* phase, int Nz, size_t plane, floa
   // without the blur only the phase is touched: the single row of CTAs takes x0 = phase
   k_constrain<V><<<grid, T, smem, st>>>(blur ? amp : phase, phase, Nz, plane, sigma, R, rz_relax, pos_relax);
   return PTY_OK;
-}
-
-// ---------------------------------------------------------------------------------------------
-// k_z filter: line transforms.  One CTA transforms C lines of length L held in shared memory:
-// radix-2 decimation in time (input stored bit-reversed, natural-order output) when L is a power
-// of two, otherwise the direct O(L^2) DFT.  Neither direction normalises.  Lines along x are rows
-// (element stride 1); lines along y are columns (stride W) taken C adjacent columns at a time, so
-// global accesses stay in contiguous runs of C (axis 1) or L (axis 0) elements.
-// ---------------------------------------------------------------------------------------------
-constexpr int kLineElems = 8192;  // C * L per CTA
-constexpr int kMaxLine = 8192;
-constexpr int kLineThreads = 256;
-
-enum LineIO { IO_Z = 0, IO_FROM_PAIR = 1, IO_TO_PAIR = 2 };
-
-struct LineArgs {
-  float2* z;     // complex volume [Nz][H][W]
-  float* amp;    // IO_FROM_PAIR: real part source; IO_TO_PAIR: destination (relaxed)
-  float* phase;  // imaginary part, likewise
-  float relax;
-  int axis;      // 0: lines along x, 1: lines along y
-  int L, C, logL, pow2;
-  int Nz, H, W;
-  int tiles_per_slice;  // axis 1: ceil(W / C)
-  long long lines;      // axis 0: Nz * H
-};
-
-// Global element of (line l of this CTA's tile, position j), or -1 when the line is past the end.
-__device__ __forceinline__ long long line_elem(const LineArgs& a, long long tile, int l, int j) {
-  if (a.axis == 0) {
-    const long long g = tile * a.C + l;
-    return g < a.lines ? g * a.W + j : -1;
-  }
-  const long long s = tile / a.tiles_per_slice;
-  const int x = (int)(tile % a.tiles_per_slice) * a.C + l;
-  return x < a.W ? (s * a.H + j) * a.W + x : -1;
-}
-
-__device__ __forceinline__ unsigned bitrev(unsigned j, int bits) { return bits ? __brev(j) >> (32 - bits) : 0u; }
-
-template <bool INV, int IO>
-__global__ void __launch_bounds__(kLineThreads) k_lines(LineArgs a) {
-  extern __shared__ __align__(16) unsigned char l_smem[];
-  const int L = a.L, C = a.C, tid = threadIdx.x;
-  const int n = C * L;
-  float2* buf = reinterpret_cast<float2*>(l_smem);  // [C][L]
-  float2* out = buf + n;                              // direct DFT: [C][L]; power of two: unused
-  float2* tw = a.pow2 ? buf + n : buf + 2 * n;        // exp(-+2 pi i t / L), t < L/2 (pow2) or < L
-  const long long tile = blockIdx.x;
-  const int ntw = a.pow2 ? L / 2 : L;
-  for (int t = tid; t < ntw; t += kLineThreads) {
-    float s, c;
-    sincospif(-2.0f * (float)t / (float)L, &s, &c);
-    tw[t] = make_float2(c, INV ? -s : s);
-  }
-  // load (contiguous runs: along j for axis 0, along l for axis 1)
-  for (int f = tid; f < n; f += kLineThreads) {
-    const int l = a.axis == 0 ? f / L : f % C;
-    const int j = a.axis == 0 ? f % L : f / C;
-    const long long e = line_elem(a, tile, l, j);
-    float2 v = make_float2(0.f, 0.f);
-    if (e >= 0) v = IO == IO_FROM_PAIR ? make_float2(a.amp[e], a.phase[e]) : a.z[e];
-    buf[l * L + (a.pow2 ? (int)bitrev((unsigned)j, a.logL) : j)] = v;
-  }
-  __syncthreads();
-  const float2* res = buf;
-  if (a.pow2) {
-    const int half = L >> 1;
-    for (int h = 1, lh = 0; h < L; h <<= 1, ++lh) {
-      for (int b = tid; b < C * half; b += kLineThreads) {
-        const int l = b / half, q = b - l * half;
-        const int r = q & (h - 1);
-        const int i = ((q >> lh) << (lh + 1)) + r;
-        const float2 w = tw[r << (a.logL - 1 - lh)];
-        float2* row = buf + l * L;
-        const float2 u = row[i], v0 = row[i + h];
-        const float2 v = make_float2(fmaf(v0.x, w.x, -v0.y * w.y), fmaf(v0.x, w.y, v0.y * w.x));
-        row[i] = make_float2(u.x + v.x, u.y + v.y);
-        row[i + h] = make_float2(u.x - v.x, u.y - v.y);
-      }
-      __syncthreads();
-    }
-  } else {
-    for (int f = tid; f < n; f += kLineThreads) {
-      const int l = f / L, k = f - l * L;
-      const float2* row = buf + l * L;
-      float2 acc = make_float2(0.f, 0.f);
-      int t = 0;  // (j * k) mod L
-      for (int j = 0; j < L; ++j) {
-        const float2 x = row[j], w = tw[t];
-        acc.x = fmaf(x.x, w.x, fmaf(-x.y, w.y, acc.x));
-        acc.y = fmaf(x.x, w.y, fmaf(x.y, w.x, acc.y));
-        t += k;
-        if (t >= L) t -= L;
-      }
-      out[f] = acc;
-    }
-    __syncthreads();
-    res = out;
-  }
-  for (int f = tid; f < n; f += kLineThreads) {
-    const int l = a.axis == 0 ? f / L : f % C;
-    const int j = a.axis == 0 ? f % L : f / C;
-    const long long e = line_elem(a, tile, l, j);
-    if (e < 0) continue;
-    const float2 v = res[l * L + j];
-    if (IO == IO_TO_PAIR) {
-      const float x0 = a.amp[e], y0 = a.phase[e];
-      a.amp[e] = x0 + a.relax * (v.x - x0);
-      a.phase[e] = y0 + a.relax * (v.y - y0);
-    } else {
-      a.z[e] = v;
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------------------------
-// k_z filter: per (k_y, k_x) column of the laterally transformed volume, the depth DFT, the
-// filter W_a (Eq. 10-11) with the 1 / (Nz H W) of the inverse 3D DFT, and the inverse depth DFT.
-// One thread per column; the column and its spectrum sit in shared memory ([Nz][T] each).
-// ---------------------------------------------------------------------------------------------
-constexpr float kKzEps = 1e-3f;  // per square angstrom, the stabilising constant under Eq. 10
-
-// DFT frequency of bin i of n samples spaced d, in cycles per unit of d (numpy's fftfreq)
-__device__ __forceinline__ float fft_freq(int i, int n, float d) {
-  return (float)(i < (n + 1) / 2 ? i : i - n) / ((float)n * d);
-}
-
-__global__ void k_kz_columns(float2* __restrict__ z, int Nz, int H, int W, float dx, const float* __restrict__ dz,
-                             float beta, float alpha) {
-  extern __shared__ __align__(16) unsigned char k_smem[];
-  const int T = blockDim.x, tid = threadIdx.x;
-  float2* tw = reinterpret_cast<float2*>(k_smem);  // exp(-2 pi i t / Nz)
-  float2* col = tw + Nz;                           // [Nz][T]
-  float2* spec = col + (size_t)Nz * T;             // [Nz][T]
-  const size_t plane = (size_t)H * W;
-  const size_t p = blockIdx.x * (size_t)T + tid;
-  for (int t = tid; t < Nz; t += T) {
-    float s, c;
-    sincospif(-2.0f * (float)t / (float)Nz, &s, &c);
-    tw[t] = make_float2(c, s);
-  }
-  const bool in = p < plane;
-  if (in)
-    for (int s = 0; s < Nz; ++s) col[(size_t)s * T + tid] = z[(size_t)s * plane + p];
-  __syncthreads();
-  if (!in) return;
-  const float kx = fft_freq((int)(p % W), W, dx), ky = fft_freq((int)(p / W), H, dx);
-  const float kr2 = kx * kx + ky * ky;
-  const float dzv = *dz;
-  const float lateral = expf(-alpha * kr2) / ((float)Nz * (float)plane);
-  const float b2 = beta * beta, den = kr2 + kKzEps;
-  for (int k = 0; k < Nz; ++k) {
-    float2 acc = make_float2(0.f, 0.f);
-    int t = 0;  // (s * k) mod Nz
-    for (int s = 0; s < Nz; ++s) {
-      const float2 x = col[(size_t)s * T + tid], w = tw[t];
-      acc.x = fmaf(x.x, w.x, fmaf(-x.y, w.y, acc.x));
-      acc.y = fmaf(x.x, w.y, fmaf(x.y, w.x, acc.y));
-      t += k;
-      if (t >= Nz) t -= Nz;
-    }
-    const float kz = fft_freq(k, Nz, dzv);
-    const float wk = (1.0f - 0.63661977236758134f * atanf(b2 * kz * kz / den)) * lateral;  // 2 / pi
-    spec[(size_t)k * T + tid] = make_float2(acc.x * wk, acc.y * wk);
-  }
-  for (int s = 0; s < Nz; ++s) {
-    float2 acc = make_float2(0.f, 0.f);
-    int t = 0;  // (s * k) mod Nz, conjugate twiddles
-    for (int k = 0; k < Nz; ++k) {
-      const float2 x = spec[(size_t)k * T + tid], w = tw[t];
-      acc.x = fmaf(x.x, w.x, fmaf(x.y, w.y, acc.x));
-      acc.y = fmaf(x.y, w.x, fmaf(-x.x, w.y, acc.y));
-      t += s;
-      if (t >= Nz) t -= Nz;
-    }
-    z[(size_t)s * plane + p] = acc;
-  }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -555,40 +374,43 @@ static int check_constraints(const pty_geom* geom, const pty_constraints* c) {
   return PTY_OK;
 }
 
-static int run_lines(LineArgs a, bool inverse, int io, cudaStream_t st) {
-  a.pow2 = (a.L & (a.L - 1)) == 0;
-  a.logL = 0;
-  while ((1 << a.logL) < a.L) ++a.logL;
-  int C = kLineElems / a.L;
-  C = C < 1 ? 1 : C > 16 ? 16 : C;
-  while (C & (C - 1)) C &= C - 1;  // a power of two
-  a.C = C;
-  const size_t n = (size_t)C * a.L;
-  const size_t smem = sizeof(float2) * (a.pow2 ? n + a.L / 2 : 2 * n + a.L);
-  long long tiles;
-  if (a.axis == 0) {
-    a.lines = (long long)a.Nz * a.H;
-    tiles = (a.lines + C - 1) / C;
-  } else {
-    a.tiles_per_slice = (a.W + C - 1) / C;
-    tiles = (long long)a.Nz * a.tiles_per_slice;
-  }
-  auto kern = io == IO_FROM_PAIR ? k_lines<false, IO_FROM_PAIR>
-            : io == IO_TO_PAIR   ? k_lines<true, IO_TO_PAIR>
-            : inverse            ? k_lines<true, IO_Z>
-                                 : k_lines<false, IO_Z>;
-  if (smem > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-                              cudaSuccess) {
-    set_error("cudaFuncSetAttribute(k_lines) failed: %s", cudaGetErrorString(cudaGetLastError()));
+template <class Kern>
+static int big_smem(Kern kern, size_t smem, const char* what) {
+  if (smem > 48 * 1024 &&
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    set_error("cudaFuncSetAttribute(%s) failed: %s", what, cudaGetErrorString(cudaGetLastError()));
     return PTY_ECUDA;
   }
-  kern<<<(unsigned)tiles, kLineThreads, smem, st>>>(a);
-  return launched("k_lines");
+  return PTY_OK;
+}
+
+// One pass of line transforms.  C lines per tile, a power of two up to 8 while two CTAs fit an SM, at least
+// one; as many CTAs as fit the chip at once take the tiles in turn.
+template <int MODE, int KIND>
+static int run_lines_of(KzArgs a, cudaStream_t st) {
+  constexpr bool X = MODE == KZ_X_FWD || MODE == KZ_X_INV;
+  const size_t tables = kz_table_bytes(a.line);
+  a.C = KIND == KZ_DIRECT ? 1 : 8;
+  while (a.C > 1 && tables + kz_lines_bytes(a.line, a.C) > kKzSmem / 2) a.C /= 2;
+  const size_t smem = tables + kz_lines_bytes(a.line, a.C);
+  a.tiles = X ? (long long)a.Nz * ((a.H + a.C - 1) / a.C) : (long long)((a.W + 7) / 8) * a.Nz * (8 / a.C);
+  int rc = big_smem(k_kz_lines<MODE, KIND>, smem, "k_kz_lines");
+  if (rc) return rc;
+  long long per_sm = (long long)(kKzSmem / (smem + 1024));
+  per_sm = per_sm < 1 ? 1 : per_sm > 4 ? 4 : per_sm;
+  const long long grid = a.tiles < 152 * per_sm ? a.tiles : 152 * per_sm;
+  k_kz_lines<MODE, KIND><<<(unsigned)grid, kKzThreads, smem, st>>>(a);
+  return launched("k_kz_lines");
+}
+template <int MODE>
+static int run_lines(const KzArgs& a, cudaStream_t st) {
+  return a.line.kind == KZ_POW2 ? run_lines_of<MODE, KZ_POW2>(a, st)
+       : a.line.kind == KZ_BLUESTEIN ? run_lines_of<MODE, KZ_BLUESTEIN>(a, st) : run_lines_of<MODE, KZ_DIRECT>(a, st);
 }
 
 static int run_kz_filter(const pty_geom* g, float* amp, float* phase, const float* dz, const pty_constraints* c,
                          float2* z, cudaStream_t st) {
-  LineArgs a;
+  KzArgs a;
   memset(&a, 0, sizeof(a));
   a.z = z;
   a.amp = amp;
@@ -597,29 +419,21 @@ static int run_kz_filter(const pty_geom* g, float* amp, float* phase, const floa
   a.Nz = g->Nz;
   a.H = g->H;
   a.W = g->W;
+  const KzLine lx = kz_line(g->W), ly = kz_line(g->H);
   int rc;
-  a.axis = 0;
-  a.L = g->W;
-  if ((rc = run_lines(a, false, IO_FROM_PAIR, st))) return rc;
-  a.axis = 1;
-  a.L = g->H;
-  if ((rc = run_lines(a, false, IO_Z, st))) return rc;
-  const size_t plane = (size_t)g->H * g->W;
-  int T = (int)((kConstrainSmem - sizeof(float2) * g->Nz) / (2 * sizeof(float2) * (size_t)g->Nz));
-  T = T >= 128 ? 128 : T / 32 * 32;
-  const size_t smem = sizeof(float2) * ((size_t)g->Nz + 2 * (size_t)g->Nz * T);
-  if (smem > 48 * 1024 && cudaFuncSetAttribute(k_kz_columns, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)smem) != cudaSuccess) {
-    set_error("cudaFuncSetAttribute(k_kz_columns) failed: %s", cudaGetErrorString(cudaGetLastError()));
-    return PTY_ECUDA;
-  }
-  k_kz_columns<<<(unsigned)((plane + T - 1) / T), T, smem, st>>>(z, g->Nz, g->H, g->W, g->dx, dz, c->kz_beta,
-                                                                 c->kz_alpha);
-  if ((rc = launched("k_kz_columns"))) return rc;
-  if ((rc = run_lines(a, true, IO_Z, st))) return rc;
-  a.axis = 0;
-  a.L = g->W;
-  return run_lines(a, true, IO_TO_PAIR, st);
+  a.line = lx;
+  if ((rc = run_lines<KZ_X_FWD>(a, st))) return rc;
+  a.line = ly;
+  if ((rc = run_lines<KZ_Y_FWD>(a, st))) return rc;
+  const size_t smem = kz_depth_bytes(g->Nz);
+  if ((rc = big_smem(k_kz_depth, smem, "k_kz_depth"))) return rc;
+  const int columns = g->H * (g->W < 8 ? g->W : 8);  // of a block
+  k_kz_depth<<<dim3((columns + kDepthThreads - 1) / kDepthThreads, (g->W + 7) / 8), kDepthThreads, smem, st>>>(
+      z, g->Nz, g->H, g->W, g->dx, dz, c->kz_beta, c->kz_alpha, lx, ly);
+  if ((rc = launched("k_kz_depth"))) return rc;
+  if ((rc = run_lines<KZ_Y_INV>(a, st))) return rc;
+  a.line = lx;
+  return run_lines<KZ_X_INV>(a, st);
 }
 
 static int run_orthogonalize(const pty_geom* g, float* probe, const ConstrainLayout& L, char* ws, cudaStream_t st) {

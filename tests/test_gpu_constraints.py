@@ -79,6 +79,25 @@ def test_kz_filter_matches_oracle(Nz, H, W, beta, alpha, relax):
         assert np.abs(g - ref).max() <= 2e-5
 
 
+# The line transforms of the filter: a narrow last block of x positions (67, 71), mixed radices, lines of
+# other lengths at 4, 2 and 1 lines a tile (up to P = 8192), the longest power of two, and the direct sum
+# past 4096; depths of one slice, not a multiple of eight, and the largest.  FP32 transforms err by a few
+# eps log2(P) < 2e-6; the direct sum of L terms by about eps sqrt(L) a line, 1e-5 with its two passes.
+@pytest.mark.parametrize("Nz,H,W,bar", [(128, 64, 67, 2e-6), (5, 256, 71, 2e-6), (9, 2048, 64, 2e-6), (3, 300, 65, 2e-6),
+                                        (2, 64, 2050, 2e-6), (1, 100, 4095, 2e-6), (1, 8192, 66, 2e-6),
+                                        (2, 64, 4097, 1e-5), (1, 4100, 65, 1e-5)])
+def test_kz_filter_line_lengths(Nz, H, W, bar):
+    from paper_2505_07814_gb300.ptycho import constrain
+    pt, params, amp, phase = _setup(Nz, H, W, seed=3 * Nz + W)
+    _with_dz(params, 2.0)
+    constrain(pt, params, kz_beta=0.8, kz_alpha=0.01, kz_relax=0.9)
+    torch.cuda.synchronize()
+    for got, x in ((params.amp, amp), (params.phase, phase)):
+        ref = K.kz_filter(x, pt.geom.dx, 2.0, 0.8, 0.01, 0.9)
+        g = got.cpu().numpy().astype(np.float64)
+        assert np.linalg.norm(g - ref) <= bar * np.linalg.norm(ref), np.linalg.norm(g - ref) / np.linalg.norm(ref)
+
+
 def test_all_object_constraints_in_order():
     from paper_2505_07814_gb300.ptycho import constrain
     pt, params, amp, phase = _setup(6, 64, 70, seed=11)
