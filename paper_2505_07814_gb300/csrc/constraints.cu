@@ -2,8 +2,9 @@
 // Sec. "Physical constraints").
 //
 //   probe orthogonalisation  k_gram (FP64 Gram-matrix partials of the probe modes), k_ortho_eig
-//                            (one warp: complex Jacobi eigensolver in FP64, modes sorted by power),
-//                            k_ortho_apply (each pixel's modes mixed by the eigenvectors, in place);
+//                            (one CTA: complex Jacobi eigensolver in FP64, disjoint rotations side by
+//                            side, modes sorted by power), k_ortho_apply (each pixel's modes mixed
+//                            by the eigenvectors, in place);
 //   k_z filter (Eq. 10-12)   kz_filter.cuh: k_kz_lines along x and y, k_kz_depth, k_kz_lines back;
 //   depth blur, positivity   k_constrain (Eq. 13 and the phase clip).
 #include <cuda_runtime.h>
@@ -140,7 +141,8 @@ static int launch_constrain(float* amp, float* phase, int Nz, size_t plane, floa
 // power lambda; each column of U is turned so that its largest-magnitude entry is real positive.
 // ---------------------------------------------------------------------------------------------
 constexpr int kMaxOrthoModes = 32;
-constexpr int kGramChunk = 1024;   // pixels per k_gram CTA
+constexpr int kGramChunk = 256;    // pixels per k_gram CTA
+constexpr int kGramTile = 128;     // pixels in shared memory at a time
 constexpr int kJacobiSweeps = 60;  // cyclic sweeps at most (convergence is quadratic; a handful suffice)
 
 __device__ __forceinline__ void pair_of(int pair, int M, int* m, int* n) {
@@ -153,161 +155,254 @@ __device__ __forceinline__ void pair_of(int pair, int M, int* m, int* n) {
   *n = i + r;
 }
 
-// partial[pair][chunk] = sum over the chunk's pixels of P_m conj(P_n), m <= n
+// partial[pair][chunk] = sum over the chunk's pixels of P_m conj(P_n), m <= n.  A CTA converts its pixels'
+// modes to FP64 once in shared memory and every thread sums one mode pair over one of `groups` shares
+// of the pixels, so the pass is bound by the FP64 units (4 products per pixel and pair); one CTA per
+// (chunk, pair) read and converted every mode M times (N = 256, M = 12: 132 us, now
+// 50).
 __global__ void __launch_bounds__(256) k_gram(const float2* __restrict__ probe, int M, int NN,
                                               double2* __restrict__ partial) {
-  __shared__ double2 red[256];
-  int m, n;
-  pair_of(blockIdx.y, M, &m, &n);
-  const float2* pm = probe + (size_t)m * NN;
-  const float2* pn = probe + (size_t)n * NN;
-  double re = 0.0, im = 0.0;
-  const int p1 = min(NN, (int)(blockIdx.x + 1) * kGramChunk);
-  for (int p = blockIdx.x * kGramChunk + threadIdx.x; p < p1; p += 256) {
-    const float2 a = pm[p], b = pn[p];
-    re += (double)a.x * b.x + (double)a.y * b.y;
-    im += (double)a.y * b.x - (double)a.x * b.y;
-  }
-  red[threadIdx.x] = make_double2(re, im);
-  __syncthreads();
-  for (int h = 128; h > 0; h >>= 1) {
-    if (threadIdx.x < h) {
-      red[threadIdx.x].x += red[threadIdx.x + h].x;
-      red[threadIdx.x].y += red[threadIdx.x + h].y;
+  extern __shared__ __align__(16) double2 g_px[];  // [kGramTile][M], then [256] partial sums
+  double2* red = g_px + (size_t)kGramTile * M;
+  const int tid = threadIdx.x, np = M * (M + 1) / 2, c0 = blockIdx.x * kGramChunk;
+  const int groups = np < 256 ? 256 / np : 1;  // np <= 528: up to three pairs a thread
+  const int grp = np < 256 ? tid / np : 0;
+  double re[3] = {0.0, 0.0, 0.0}, im[3] = {0.0, 0.0, 0.0};
+  int pm[3], pn[3], cnt = 0;
+  for (int p = np < 256 ? tid % np : tid; p < np && cnt < 3 && grp < groups; p += np < 256 ? np : 256, ++cnt)
+    pair_of(p, M, &pm[cnt], &pn[cnt]);
+  for (int t0 = c0; t0 < min(NN, c0 + kGramChunk); t0 += kGramTile) {
+    __syncthreads();
+    for (int e = tid; e < kGramTile * M; e += 256) {
+      const int m = e / kGramTile, p = e % kGramTile;
+      const float2 v = t0 + p < NN ? probe[(size_t)m * NN + t0 + p] : make_float2(0.f, 0.f);
+      g_px[p * M + m] = make_double2(v.x, v.y);
     }
     __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      if (k >= cnt) break;
+      for (int p = grp; p < kGramTile; p += groups) {
+        const double2 x = g_px[p * M + pm[k]], y = g_px[p * M + pn[k]];
+        re[k] = fma(x.y, y.y, fma(x.x, y.x, re[k]));
+        im[k] = fma(-x.x, y.y, fma(x.y, y.x, im[k]));
+      }
+    }
   }
-  if (threadIdx.x == 0) partial[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = red[0];
+  if (np >= 256) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      if (k < cnt) partial[(size_t)(tid + 256 * k) * gridDim.x + blockIdx.x] = make_double2(re[k], im[k]);
+    return;
+  }
+  red[tid] = make_double2(re[0], im[0]);
+  __syncthreads();
+  if (tid < np) {
+    double2 t = red[tid];
+    for (int g = 1; g < groups; ++g) {
+      t.x += red[g * np + tid].x;
+      t.y += red[g * np + tid].y;
+    }
+    partial[(size_t)tid * gridDim.x + blockIdx.x] = t;
+  }
 }
 
 __device__ __forceinline__ double2 zmul(double2 a, double2 b) {
   return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 __device__ __forceinline__ double2 zlin(double a, double2 x, double2 b, double2 y) {  // a x + b y
-  const double2 by = zmul(b, y);
-  return make_double2(a * x.x + by.x, a * x.y + by.y);
+  return make_double2(fma(a, x.x, fma(b.x, y.x, -b.y * y.y)), fma(a, x.y, fma(b.x, y.y, b.y * y.x)));
 }
 
-// One warp: reduce the Gram partials, diagonalise with cyclic complex Jacobi rotations in FP64,
-// sort, fix the phases; writes U (column k = eigenvector of the k-th largest power) and lambda.
-__global__ void __launch_bounds__(32) k_ortho_eig(const double2* __restrict__ partial, int M, int chunks,
-                                                   double2* __restrict__ Uout, double* __restrict__ lam_out) {
+// One CTA: reduce the Gram partials, diagonalise with cyclic complex Jacobi rotations in FP64, sort,
+// fix the phases; writes U (column k = eigenvector of the k-th largest power) and lambda.
+// A sweep is M - 1 rounds of a round-robin tournament (M even; an odd M sits one mode out): a round's
+// M / 2 rotations touch disjoint mode pairs, so they run side by side.  What bounds it is the chain of FP64
+// operations of a round (an FP64 instruction occupies a scheduler for many clocks, however few of its
+// lanes are live), so a thread forms one entry of one 2 x 2 block, the rotations come from two reciprocal
+// square roots, and V follows G one round behind on the warps that would wait for them.  One rotation after the
+// other by one warp took 1.10 ms at M = 12; this 0.18-0.20.
+__global__ void __launch_bounds__(256) k_ortho_eig(const double2* __restrict__ partial, int M, int chunks,
+                                                    double2* __restrict__ Uout, double* __restrict__ lam_out) {
+  constexpr int kMaxPairs = kMaxOrthoModes / 2;
   __shared__ double2 G[kMaxOrthoModes][kMaxOrthoModes + 1];
   __shared__ double2 V[kMaxOrthoModes][kMaxOrthoModes + 1];
   __shared__ double lam[kMaxOrthoModes];
-  const int lane = threadIdx.x;
+  __shared__ double rc[2][kMaxPairs];  // this round's rotations and the last one's (V follows a round behind)
+  __shared__ double2 rs[2][kMaxPairs];
+  __shared__ int rp[2][kMaxPairs], rq[2][kMaxPairs];
+  __shared__ int done;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int npairs = M * (M + 1) / 2;
-  for (int pr = lane; pr < npairs; pr += 32) {
+  for (int pr = warp; pr < npairs; pr += 8) {
     int m, n;
     pair_of(pr, M, &m, &n);
-    double re = 0.0, im = 0.0;
-    for (int c = 0; c < chunks; ++c) {
+    double x = 0.0, y = 0.0;
+    for (int c = lane; c < chunks; c += 32) {
       const double2 v = partial[(size_t)pr * chunks + c];
-      re += v.x;
-      im += v.y;
-    }
-    G[m][n] = make_double2(re, im);
-    G[n][m] = make_double2(re, -im);
-  }
-  if (lane < M)
-    for (int j = 0; j < M; ++j) V[lane][j] = make_double2(lane == j ? 1.0 : 0.0, 0.0);
-  __syncwarp();
-  for (int sweep = 0; sweep < kJacobiSweeps; ++sweep) {
-    double off = 0.0, diag = 0.0;
-    for (int i = lane; i < M; i += 32) {
-      diag += G[i][i].x * G[i][i].x;
-      for (int j = i + 1; j < M; ++j) off += G[i][j].x * G[i][j].x + G[i][j].y * G[i][j].y;
+      x += v.x;
+      y += v.y;
     }
     for (int o = 16; o > 0; o >>= 1) {
-      off += __shfl_xor_sync(0xffffffffu, off, o);
-      diag += __shfl_xor_sync(0xffffffffu, diag, o);
+      x += __shfl_xor_sync(0xffffffffu, x, o);
+      y += __shfl_xor_sync(0xffffffffu, y, o);
     }
-    if (!(off > 1e-30 * diag)) break;  // also ends on an all-zero matrix
-    for (int p = 0; p < M - 1; ++p) {
-      for (int q = p + 1; q < M; ++q) {
-        const double2 g = G[p][q];
-        const double ag = sqrt(g.x * g.x + g.y * g.y);
-        const double app = G[p][p].x, aqq = G[q][q].x;
-        if (!(ag > 1e-290)) continue;  // already zero (or denormal)
-        const double tau = (aqq - app) / (2.0 * ag);
-        const double t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-        const double c = 1.0 / sqrt(1.0 + t * t), s = t * c;
-        const double2 e = make_double2(g.x / ag, g.y / ag);    // e^{i phi}
-        const double2 ec = make_double2(e.x, -e.y);              // e^{-i phi}
-        const double2 mse = make_double2(-s * ec.x, -s * ec.y);  // -s e^{-i phi}
-        const double2 cec = make_double2(c * ec.x, c * ec.y);    // c e^{-i phi}
-        __syncwarp();
-        // columns p, q of G and V: X <- X U with U_pp = c, U_pq = s, U_qp = -s e^{-i phi}, U_qq = c e^{-i phi}
-        if (lane < M) {
-          const double2 gp = G[lane][p], gq = G[lane][q];
-          G[lane][p] = zlin(c, gp, mse, gq);
-          G[lane][q] = zlin(s, gp, cec, gq);
-          const double2 vp = V[lane][p], vq = V[lane][q];
-          V[lane][p] = zlin(c, vp, mse, vq);
-          V[lane][q] = zlin(s, vp, cec, vq);
-        }
-        __syncwarp();
-        // rows p, q of G: G <- U^H G
-        if (lane < M) {
-          const double2 gp = G[p][lane], gq = G[q][lane];
-          G[p][lane] = zlin(c, gp, make_double2(-s * e.x, -s * e.y), gq);
-          G[q][lane] = zlin(s, gp, make_double2(c * e.x, c * e.y), gq);
-        }
-        __syncwarp();
-        if (lane == 0) {
-          G[p][q] = make_double2(0.0, 0.0);
-          G[q][p] = make_double2(0.0, 0.0);
-          G[p][p].y = 0.0;
-          G[q][q].y = 0.0;
-        }
-        __syncwarp();
-      }
+    if (lane == 0) {
+      G[m][n] = make_double2(x, m == n ? 0.0 : y);
+      G[n][m] = make_double2(x, m == n ? 0.0 : -y);
     }
   }
-  if (lane < M) lam[lane] = G[lane][lane].x;
-  __syncwarp();
-  if (lane < M) {
+  for (int i = tid; i < M * M; i += 256) V[i / M][i % M] = make_double2(i / M == i % M ? 1.0 : 0.0, 0.0);
+  __syncthreads();
+  const int n = (M + 1) & ~1, half = n / 2, tri = half * (half + 1) / 2;
+  const double2 zero = make_double2(0.0, 0.0);
+  // V <- V U for the rotations in slot k; the two threads of a pair of entries are neighbours, t0 a warp's
+  // multiple of 32
+  auto turn_v = [&](int k, int t0, int step) {
+    for (int b = t0 + lane; b < (2 * M * half + 31) / 32 * 32; b += step) {
+      const int row = b / 2 / half, j = b / 2 % half, d = b & 1;
+      const bool on = row < M && rq[k][j] < M;  // the mode that sits out is left alone
+      const int p = rp[k][j], q = rq[k][j];
+      double2 v = zero;
+      if (on) {
+        const double2 s = rs[k][j], vp = V[row][p], vq = V[row][q];
+        v = zlin(rc[k][j], d ? vq : vp, make_double2(d ? s.x : -s.x, s.y), d ? vp : vq);
+      }
+      __syncwarp();
+      if (on) V[row][d ? q : p] = v;
+    }
+  };
+  int rounds = 0;
+  for (int sweep = 0; sweep < kJacobiSweeps; ++sweep) {
+    if (warp == 0) {
+      double off = 0.0, diag = 0.0;
+      for (int i = lane; i < M; i += 32) {
+        diag += G[i][i].x * G[i][i].x;
+        for (int j = i + 1; j < M; ++j) off += G[i][j].x * G[i][j].x + G[i][j].y * G[i][j].y;
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        off += __shfl_xor_sync(0xffffffffu, off, o);
+        diag += __shfl_xor_sync(0xffffffffu, diag, o);
+      }
+      if (lane == 0) done = !(off > 1e-30 * diag);  // also ends on an all-zero matrix
+    }
+    __syncthreads();
+    if (done) break;
+    for (int r = 0; r < n - 1; ++r, ++rounds) {
+      const int k = rounds & 1;
+      if (warp == 0) {  // rotation `lane` of the round: the modes that meet at this table
+        if (lane < half) {
+          int p = lane == 0 ? n - 1 : (r + lane) % (n - 1), q = lane == 0 ? r : (r - lane + n - 1) % (n - 1);
+          if (p > q) {
+            const int t = p;
+            p = q;
+            q = t;
+          }
+          // c and the complex s of U_pp = U_qq = c, U_pq = s, U_qp = -conj(s), which zeroes g = G_pq.  With
+          // d = G_qq - G_pp and r = sqrt(d^2 + 4 |g|^2): c^2 = (1 + |d| / r) / 2, s = sign(d) g / (r c)
+          double c = 1.0;
+          double2 s = zero;
+          if (q < M) {
+            const double2 g = G[p][q];
+            const double g2 = fma(g.x, g.x, g.y * g.y), d = G[q][q].x - G[p][p].x, r2 = fma(d, d, 4.0 * g2);
+            if (g2 > 1e-290) {  // else g is zero (or its square is denormal)
+              const double ir = rsqrt(r2), c2 = fma(0.5 * fabs(d), ir, 0.5), ic = rsqrt(c2);
+              const double f = (d >= 0.0 ? ir : -ir) * ic;
+              c = c2 * ic;
+              s = make_double2(g.x * f, g.y * f);
+            }
+          }
+          rp[k][lane] = p;
+          rq[k][lane] = q;
+          rc[k][lane] = c;
+          rs[k][lane] = s;
+        }
+      } else if (warp >= 3 && rounds > 0) {
+        turn_v(k ^ 1, 32 * (warp - 3), 32 * 5);
+      }
+      __syncthreads();
+      // G <- U^H G U, one thread per entry of the 2 x 2 blocks (rows of rotation i, columns of rotation j, i <= j),
+      // the four of a block neighbours in one warp; blocks below the diagonal get the conjugates
+      for (int b = tid; b < (4 * tri + 31) / 32 * 32; b += 256) {
+        const bool in = b < 4 * tri;
+        const int a = (b >> 1) & 1, d = b & 1;
+        int i = 0, j = 0;
+        if (in) pair_of(b >> 2, half, &i, &j);
+        const int p = rp[k][j], q = rq[k][j], ip = rp[k][i], iq = rq[k][i];
+        const bool okc = q < M, okr = iq < M;
+        const bool on = in && (d ? okc : true) && (a ? okr : true);
+        double2 g = zero;
+        if (on) {
+          const double2 b00 = G[ip][p], b01 = okc ? G[ip][q] : zero, b10 = okr ? G[iq][p] : zero,
+                        b11 = okc && okr ? G[iq][q] : zero;
+          const double c = rc[k][j], ci = rc[k][i];
+          const double2 s = rs[k][j], si = rs[k][i], m = make_double2(d ? s.x : -s.x, s.y);
+          const double2 x = zlin(c, d ? b01 : b00, m, d ? b00 : b01), y = zlin(c, d ? b11 : b10, m, d ? b10 : b11);
+          g = zlin(ci, a ? y : x, make_double2(a ? si.x : -si.x, -si.y), a ? x : y);
+          if (i == j) {  // the rotation's own block: exactly diagonal and real
+            g.y = 0.0;
+            if (a != d) g.x = 0.0;
+          }
+        }
+        __syncwarp();
+        if (on) {
+          const int row = a ? iq : ip, col = d ? q : p;
+          G[row][col] = g;
+          if (i != j) G[col][row] = make_double2(g.x, -g.y);
+        }
+      }
+      __syncthreads();
+    }
+  }
+  if (rounds > 0) turn_v((rounds - 1) & 1, 32 * warp, 256);
+  if (tid < M) lam[tid] = G[tid][tid].x;
+  __syncthreads();
+  if (tid < M) {
     // rank of this eigenpair by decreasing power (ties keep the index order)
-    const double lk = lam[lane];
+    const double lk = lam[tid];
     int rank = 0;
-    for (int j = 0; j < M; ++j) rank += (lam[j] > lk) || (lam[j] == lk && j < lane);
+    for (int j = 0; j < M; ++j) rank += (lam[j] > lk) || (lam[j] == lk && j < tid);
     int mstar = 0;
     double best = -1.0;
     for (int m = 0; m < M; ++m) {
-      const double a = V[m][lane].x * V[m][lane].x + V[m][lane].y * V[m][lane].y;
+      const double a = V[m][tid].x * V[m][tid].x + V[m][tid].y * V[m][tid].y;
       if (a > best) {
         best = a;
         mstar = m;
       }
     }
-    const double2 vs = V[mstar][lane];
+    const double2 vs = V[mstar][tid];
     const double av = sqrt(vs.x * vs.x + vs.y * vs.y);
     const double2 ph = av > 0.0 ? make_double2(vs.x / av, -vs.y / av) : make_double2(1.0, 0.0);
-    for (int m = 0; m < M; ++m) Uout[(size_t)m * M + rank] = zmul(V[m][lane], ph);
+    for (int m = 0; m < M; ++m) Uout[(size_t)m * M + rank] = zmul(V[m][tid], ph);
     lam_out[rank] = lk;
   }
 }
 
-// Q_k[p] = sum_m conj(U[m][k]) P_m[p], in place; one thread per pixel, its M modes in shared memory.
+// Q_k[p] = sum_m conj(U[m][k]) P_m[p], in place; one thread per pixel, its M modes in shared memory, converted
+// to FP64 once (bound by the FP64 units: 4 M^2 products per pixel; N = 256, M = 12: 170 us
+// before, now 81).
 __global__ void __launch_bounds__(128) k_ortho_apply(float2* __restrict__ probe, int M, int NN,
                                                       const double2* __restrict__ U) {
   extern __shared__ __align__(16) unsigned char o_smem[];
-  double2* u = reinterpret_cast<double2*>(o_smem);                 // [M][M]
-  float2* px = reinterpret_cast<float2*>(u + (size_t)M * M);     // [M][128]
+  double2* u = reinterpret_cast<double2*>(o_smem);  // [M][M]
+  double2* px = u + (size_t)M * M;                  // [M][128]
   const int tid = threadIdx.x;
   for (int i = tid; i < M * M; i += 128) u[i] = U[i];
   const int p = blockIdx.x * 128 + tid;
   if (p < NN)
-    for (int m = 0; m < M; ++m) px[m * 128 + tid] = probe[(size_t)m * NN + p];
+    for (int m = 0; m < M; ++m) {
+      const float2 v = probe[(size_t)m * NN + p];
+      px[m * 128 + tid] = make_double2(v.x, v.y);
+    }
   __syncthreads();
   if (p >= NN) return;
   for (int k = 0; k < M; ++k) {
     double re = 0.0, im = 0.0;
     for (int m = 0; m < M; ++m) {
-      const double2 w = u[m * M + k];  // conj(w) * x
-      const float2 x = px[m * 128 + tid];
-      re += w.x * x.x + w.y * x.y;
-      im += w.x * x.y - w.y * x.x;
+      const double2 w = u[m * M + k], x = px[m * 128 + tid];  // conj(w) * x
+      re = fma(w.y, x.y, fma(w.x, x.x, re));
+      im = fma(-w.y, x.x, fma(w.x, x.y, im));
     }
     probe[(size_t)k * NN + p] = make_float2((float)re, (float)im);
   }
@@ -444,11 +539,14 @@ static int run_orthogonalize(const pty_geom* g, float* probe, const ConstrainLay
   double* lam = reinterpret_cast<double*>(ws + L.lam);
   float2* P = reinterpret_cast<float2*>(probe);
   int rc;
-  k_gram<<<dim3(chunks, M * (M + 1) / 2), 256, 0, st>>>(P, M, NN, partial);
+  const size_t gram_smem = sizeof(double2) * ((size_t)kGramTile * M + 256);
+  if ((rc = big_smem(k_gram, gram_smem, "k_gram"))) return rc;
+  k_gram<<<chunks, 256, gram_smem, st>>>(P, M, NN, partial);
   if ((rc = launched("k_gram"))) return rc;
-  k_ortho_eig<<<1, 32, 0, st>>>(partial, M, chunks, U, lam);
+  k_ortho_eig<<<1, 256, 0, st>>>(partial, M, chunks, U, lam);
   if ((rc = launched("k_ortho_eig"))) return rc;
-  const size_t smem = sizeof(double2) * M * M + sizeof(float2) * M * 128;
+  const size_t smem = sizeof(double2) * ((size_t)M * M + (size_t)M * 128);
+  if ((rc = big_smem(k_ortho_apply, smem, "k_ortho_apply"))) return rc;
   k_ortho_apply<<<(NN + 127) / 128, 128, smem, st>>>(P, M, NN, U);
   return launched("k_ortho_apply");
 }
