@@ -293,15 +293,14 @@ __global__ void __launch_bounds__(256) k_stage(StageArgs g) {
   const int b = bm / (a.M * a.Ko), m = (bm / a.Ko) % a.M;  // waves: (position, probe mode, object mode)
   const int j = checked_index(a.idx, b, a.Ntot, a.status);
   int i0, i1;
-  float d0, d1, th0, th1;
+  float d0, d1;
   patch_corner<N>(a.pos, j, a.H, a.W, &i0, &i1, &d0, &d1, a.status);
-  tilt_of(a.tilt, a.global_tilt, j, &th0, &th1);
-  const float dz = a.dz[0];
+  const Pair* wc = a.wc + (size_t)b * kWaveConsts;
   constexpr bool kAdj = ST >= GS_FARGRAD;
   if (kAdj) {
-    adj_tables<N>(t0p, t1p, t2p, t3p, e0, e1, c0, c1, f0, f1, d0, d1, th0, th1, dz, a.dx, a.lam);
+    adj_tables<N>(t0p, t1p, t2p, t3p, e0, e1, c0, c1, f0, f1, d0, d1, wc);
   } else {
-    fwd_tables<N>(t0p, t1p, t2p, t3p, d0, d1, th0, th1, dz, a.dx, a.lam);
+    fwd_tables<N>(t0p, t1p, t2p, t3p, d0, d1, wc);
   }
   __syncthreads();
   const size_t plane = (size_t)a.H * a.W, patch = (size_t)(bm % a.Ko) * a.Nz * plane + (size_t)i0 * a.W + i1;

@@ -3,7 +3,8 @@
 // loop; the wave never leaves shared memory except as checkpoints for the adjoint.
 //
 // Kernel sequence of one pty_loss_grad call (one stream, no host synchronisation):
-//   k_prepare_object   T = amp exp(i phase) for the whole object; zero dL/dT accumulator
+//   k_prepare          T = amp exp(i phase) for the whole object; the constants of every batch
+//                      entry's tables
 //   k_probe_spectrum   P^_m = F[P_m]                                              (M CTAs)
 //   k_forward          shift, Nz transmissions, Nz-1 propagations, far field      (B*M CTAs)
 //   k_loss             mode sum, Eq. 5/6 per pixel, dL/dI, per-pattern sums      (B CTAs)
@@ -167,12 +168,38 @@ __host__ __device__ constexpr int wave_rows() {
   return N == 256 ? 256 / PTY_N256_CTAS : N;
 }
 
-// exp(i pi x); x is reduced modulo 2 in double precision before the float sincospi.
-__device__ __forceinline__ float2 expipi(double x) {
-  x = x - 2.0 * rint(0.5 * x);
+// A real number as an unevaluated sum of two floats (48 significant bits).  The per-wave tables are built with
+// pairs of floats instead of FP64: an FP64 instruction occupies a scheduler for 64 clocks here, and the
+// tables' divisions, tangents and cosines in FP64 took 6.5 us (forward) and 13 us (adjoint) of every wave.
+struct Pair {
+  float hi, lo;
+};
+__device__ __forceinline__ Pair to_pair(double x) {
+  const float h = (float)x;
+  return Pair{h, (float)(x - (double)h)};
+}
+// q2 a + q b for integers |q| <= 128 and q2 = q^2 (exact in float); the roundings are kept in lo
+__device__ __forceinline__ Pair pair_poly(float q2, Pair a, float q, Pair b) {
+  const float p = __fmul_rn(q2, a.hi), r = __fmul_rn(q, b.hi);
+  const float pe = fmaf(q2, a.hi, -p), re = fmaf(q, b.hi, -r);
+  const float s = __fadd_rn(p, r), t = __fadd_rn(s, -p);
+  const float e = __fadd_rn(__fadd_rn(p, -__fadd_rn(s, -t)), __fadd_rn(r, -t));
+  return Pair{s, e + pe + re + fmaf(q2, a.lo, q * b.lo)};
+}
+__device__ __forceinline__ float pair_value(Pair a) { return a.hi + a.lo; }
+// exp(i pi (hi + lo)): hi reduced modulo 2 exactly, lo as a first-order rotation
+__device__ __forceinline__ float2 expipi(Pair x) {
+  const float r = x.hi - 2.0f * rintf(0.5f * x.hi);
   float s, c;
-  sincospif((float)x, &s, &c);
-  return make_float2(c, s);
+  sincospif(r, &s, &c);
+  const float d = 3.14159265358979f * x.lo;
+  return make_float2(fmaf(-d, s, c), fmaf(d, c, s));
+}
+// exp(i pi f q d / N) for f = +-2: the shift ramp of bin q for a sub-pixel shift |d| <= 1/2
+template <int N>
+__device__ __forceinline__ float2 ramp(float f, float q, float d) {
+  const float p = __fmul_rn(q, d), w = f / (float)N;  // w: a power of two
+  return expipi(Pair{p * w, fmaf(q, d, -p) * w});
 }
 
 // Signed DFT frequency index of bin k.
@@ -216,23 +243,58 @@ __device__ __forceinline__ int checked_index(const int32_t* idx, int b, int Ntot
   return j;
 }
 
-__device__ __forceinline__ void tilt_of(const float* tilt, int global_tilt, int j, float* t0, float* t1) {
-  const float* t = global_tilt ? tilt : tilt + 2 * j;
-  *t0 = t[0];
-  *t1 = t[1];
-}
+// Constants of one batch entry's tables, formed once per call (FP64, then pairs of floats): with k = q kq for
+// signed bin q and kq = 1 / (N dx), the propagator's phase over pi is q^2 K2 + q K_a, its dz derivative
+// q^2 E2 + q E_a, its tilt derivative q C_a (signs of AdjPropStore's terms).
+enum { WC_K2, WC_K0, WC_K1, WC_E2, WC_E0, WC_E1, WC_C0, WC_C1, kWaveConsts };
+static_assert(kWaveConsts * 2 == kWaveConstFloats, "workspace layout");
 
 // ---------------------------------------------------------------------------------------------
-// Object transmission and accumulator reset
+// Start of a forward: object transmission (blocks 0 .. blocks - 1) and, by the blocks after them, the
+// constants of every batch entry, four threads an entry (its tangents and cosines are chains of some
+// hundred FP64 instructions, so each has a thread of its own).
 // ---------------------------------------------------------------------------------------------
-static __global__ void k_prepare_object(const float* __restrict__ amp, const float* __restrict__ phase,
-                                 float2* __restrict__ T, float2* __restrict__ gT, size_t n) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+struct PrepArgs {
+  const float *amp, *phase;
+  float2* T;
+  size_t n;
+  int blocks;  // of the object part
+  int B, Ntot, global_tilt;
+  double lam, kq;
+  const int32_t* idx;
+  const float *tilt, *dz;
+  Pair* wc;  // [B][kWaveConsts]
+  int* status;
+};
+static __global__ void __launch_bounds__(256) k_prepare(PrepArgs a) {
+  if ((int)blockIdx.x >= a.blocks) {
+    const int t = (blockIdx.x - a.blocks) * 256 + threadIdx.x, part = t / 32 & 3, b = (t / 128) * 32 + (t & 31);
+    if (b >= a.B) return;
+    int j = a.idx[b];
+    if (j < 0 || j >= a.Ntot) {
+      atomicOr(a.status, PTY_EBOUNDS);
+      j = 0;
+    }
+    const float* th = a.global_tilt ? a.tilt : a.tilt + 2 * (size_t)j;
+    const double PI = 3.14159265358979323846, dz = a.dz[0], x = (double)th[part & 1];
+    Pair* w = a.wc + (size_t)b * kWaveConsts;
+    if (part < 2) {
+      const double tn = tan(x);
+      w[WC_K0 + part] = to_pair(2.0 * dz * tn * a.kq);
+      w[WC_E0 + part] = to_pair(-2.0 * PI * tn * a.kq);
+    } else {
+      const double c = cos(x);
+      w[WC_C0 + part - 2] = to_pair(-2.0 * PI * dz * a.kq / (c * c));
+      if (part == 2) w[WC_K2] = to_pair(-a.lam * dz * a.kq * a.kq);
+      else w[WC_E2] = to_pair(PI * a.lam * a.kq * a.kq);
+    }
+    return;
+  }
+  for (size_t i = blockIdx.x * (size_t)256 + threadIdx.x; i < a.n; i += (size_t)a.blocks * 256) {
     float s, c;
-    sincosf(phase[i], &s, &c);
-    const float a = amp[i];
-    T[i] = make_float2(a * c, a * s);
-    if (gT) gT[i] = make_float2(0.f, 0.f);
+    sincosf(a.phase[i], &s, &c);
+    const float m = a.amp[i];
+    a.T[i] = make_float2(m * c, m * s);
   }
 }
 
@@ -266,10 +328,10 @@ __global__ void __launch_bounds__(T) k_probe_spectrum(const float2* __restrict__
 // Forward: one CTA per (batch entry b, mode m)
 // ---------------------------------------------------------------------------------------------
 struct FwdArgs {
-  int M, Ko, Nz, H, W, Ntot, global_tilt;  // Ko: object modes
-  float dx, lam;
+  int M, Ko, Nz, H, W, Ntot;  // Ko: object modes
   const int32_t* idx;
-  const float *pos, *tilt, *dz;
+  const float* pos;
+  const Pair* wc;  // [batch entry][kWaveConsts]
   const float2* T;
   const float2* Phat;
   float2* ckpt;     // every slice's entering wave [wave][Nz][N*N], or nullptr
@@ -422,44 +484,39 @@ __device__ __forceinline__ bool stage_wait(uint32_t bar, uint32_t parity) {
 // tables by k-space column p1).  Forward: shift ramps R (axis 0 carries the 1/N^2 of the inverse
 // DFT) and the two factors of Eq. 4's propagator (axis 0 carries 1/N^2).
 template <int N>
-__device__ void fwd_tables(float2* ra0, float2* ra1, float2* pm0, float2* pm1, float d0, float d1, float th0, float th1,
-                           float dz, float dx, float lam) {
+__device__ void fwd_tables(float2* ra0, float2* ra1, float2* pm0, float2* pm1, float d0, float d1,
+                           const Pair* __restrict__ wc) {
   for (int tid = threadIdx.x; tid < N; tid += blockDim.x) {
-    const int q0 = signed_bin<N>(kbin0<N>(tid)), q1 = signed_bin<N>(kbin1<N>(tid));
+    const float q0 = (float)signed_bin<N>(kbin0<N>(tid)), q1 = (float)signed_bin<N>(kbin1<N>(tid));
     const float inv_nn = 1.0f / (float)(N * N);
-    ra0[tid] = cscale(expipi(-2.0 * q0 * (double)d0 / N), inv_nn);
-    ra1[tid] = expipi(-2.0 * q1 * (double)d1 / N);
+    ra0[tid] = cscale(ramp<N>(-2.0f, q0, d0), inv_nn);
+    ra1[tid] = ramp<N>(-2.0f, q1, d1);
     // Eq. 4 split into its two axes: exp(i pi (-lam dz k_a^2 + 2 dz k_a tan th_a))
-    const double k0 = q0 / (N * (double)dx), k1 = q1 / (N * (double)dx);
-    pm0[tid] = cscale(expipi(-(double)lam * dz * k0 * k0 + 2.0 * dz * k0 * tan((double)th0)), inv_nn);
-    pm1[tid] = expipi(-(double)lam * dz * k1 * k1 + 2.0 * dz * k1 * tan((double)th1));
+    pm0[tid] = cscale(expipi(pair_poly(q0 * q0, wc[WC_K2], q0, wc[WC_K0])), inv_nn);
+    pm1[tid] = expipi(pair_poly(q1 * q1, wc[WC_K2], q1, wc[WC_K1]));
   }
 }
 // Adjoint: conjugate propagator factors (axis 0 with 1/N^2), conjugate shift ramps, and the real
 // factors of the dz, tilt and position terms (signs and 2 pi / N^2 folded in).
 template <int N>
 __device__ void adj_tables(float2* cm0, float2* cm1, float2* cr0, float2* cr1, float* e0, float* e1, float* c0,
-                           float* c1, float* f0, float* f1, float d0, float d1, float th0, float th1, float dz,
-                           float dx, float lam) {
-  constexpr int NN = N * N;
+                           float* c1, float* f0, float* f1, float d0, float d1, const Pair* __restrict__ wc) {
+  constexpr double kF = 2.0 * 3.14159265358979323846 / ((double)N * N * N);
+  constexpr float kFhi = (float)kF, kFlo = (float)(kF - (double)kFhi);
   for (int tid = threadIdx.x; tid < N; tid += blockDim.x) {
     // axis-0 tables are indexed by k-space row p0, axis-1 tables by k-space column p1
-    const int q0 = signed_bin<N>(kbin0<N>(tid)), q1 = signed_bin<N>(kbin1<N>(tid));
-    const float inv_nn = 1.0f / (float)NN;
-    const double k0 = q0 / (N * (double)dx), k1 = q1 / (N * (double)dx);
-    const double tn0 = tan((double)th0), tn1 = tan((double)th1);
-    cm0[tid] = cscale(cconj(expipi(-(double)lam * dz * k0 * k0 + 2.0 * dz * k0 * tn0)), inv_nn);
-    cm1[tid] = cconj(expipi(-(double)lam * dz * k1 * k1 + 2.0 * dz * k1 * tn1));
-    cr0[tid] = expipi(2.0 * q0 * (double)d0 / N);
-    cr1[tid] = expipi(2.0 * q1 * (double)d1 / N);
-    const double PI = 3.14159265358979323846;
-    const double cs0 = cos((double)th0), cs1 = cos((double)th1);
-    e0[tid] = (float)(PI * lam * k0 * k0 - 2.0 * PI * k0 * tn0);
-    e1[tid] = (float)(PI * lam * k1 * k1 - 2.0 * PI * k1 * tn1);
-    c0[tid] = (float)(-2.0 * PI * dz * k0 / (cs0 * cs0));
-    c1[tid] = (float)(-2.0 * PI * dz * k1 / (cs1 * cs1));
-    f0[tid] = (float)(2.0 * PI * q0 / ((double)N * NN));
-    f1[tid] = (float)(2.0 * PI * q1 / ((double)N * NN));
+    const float q0 = (float)signed_bin<N>(kbin0<N>(tid)), q1 = (float)signed_bin<N>(kbin1<N>(tid));
+    const float inv_nn = 1.0f / (float)(N * N);
+    cm0[tid] = cscale(cconj(expipi(pair_poly(q0 * q0, wc[WC_K2], q0, wc[WC_K0]))), inv_nn);
+    cm1[tid] = cconj(expipi(pair_poly(q1 * q1, wc[WC_K2], q1, wc[WC_K1])));
+    cr0[tid] = ramp<N>(2.0f, q0, d0);
+    cr1[tid] = ramp<N>(2.0f, q1, d1);
+    e0[tid] = pair_value(pair_poly(q0 * q0, wc[WC_E2], q0, wc[WC_E0]));
+    e1[tid] = pair_value(pair_poly(q1 * q1, wc[WC_E2], q1, wc[WC_E1]));
+    c0[tid] = fmaf(q0, wc[WC_C0].hi, q0 * wc[WC_C0].lo);
+    c1[tid] = fmaf(q1, wc[WC_C1].hi, q1 * wc[WC_C1].lo);
+    f0[tid] = fmaf(q0, kFhi, q0 * kFlo);
+    f1[tid] = fmaf(q1, kFhi, q1 * kFlo);
   }
 }
 
@@ -579,10 +636,8 @@ __global__ void __launch_bounds__(T, Launch<N>::MINB_F) k_forward(FwdArgs a) {
   const int b = bm / (a.M * Ko), m = (bm / Ko) % a.M;  // waves: (position, probe mode, object mode)
   const int j = checked_index(a.idx, b, a.Ntot, a.status);
   int i0, i1;
-  float d0, d1, th0, th1;
+  float d0, d1;
   patch_corner<N>(a.pos, j, a.H, a.W, &i0, &i1, &d0, &d1, a.status);
-  tilt_of(a.tilt, a.global_tilt, j, &th0, &th1);
-  const float dz = a.dz[0];
   const size_t plane = (size_t)a.H * a.W;
   const float2* Tpatch = a.T + (OM ? (size_t)(bm % Ko) * a.Nz * plane : 0) + (size_t)i0 * a.W + i1;
 #if PTY_FWD_PF
@@ -621,7 +676,7 @@ __global__ void __launch_bounds__(T, Launch<N>::MINB_F) k_forward(FwdArgs a) {
   }
 
   build_twiddles<N>(tw);
-  fwd_tables<N>(ra0, ra1, pm0, pm1, d0, d1, th0, th1, dz, a.dx, a.lam);
+  fwd_tables<N>(ra0, ra1, pm0, pm1, d0, d1, a.wc + (size_t)b * kWaveConsts);
   __syncthreads();
 
   // Shifted probe P_j = F^-1[P^_m R]: the row and block steps of the inverse here; its column step
@@ -736,15 +791,13 @@ __global__ void __launch_bounds__(T, Launch<N>::MINB_F) k_recompute(FwdArgs a) {
   const int b = bm / (a.M * Ko), m = (bm / Ko) % a.M;  // waves: (position, probe mode, object mode)
   const int j = checked_index(a.idx, b, a.Ntot, a.status);
   int i0, i1;
-  float d0, d1, th0, th1;
+  float d0, d1;
   patch_corner<N>(a.pos, j, a.H, a.W, &i0, &i1, &d0, &d1, a.status);
-  tilt_of(a.tilt, a.global_tilt, j, &th0, &th1);
-  const float dz = a.dz[0];
   const size_t plane = (size_t)a.H * a.W;
   const float2* Tpatch = a.T + (OM ? (size_t)(bm % Ko) * a.Nz * plane : 0) + (size_t)i0 * a.W + i1;
   const int K = a.kstride;
   build_twiddles<N>(tw);
-  fwd_tables<N>(ra0, ra1, pm0, pm1, d0, d1, th0, th1, dz, a.dx, a.lam);
+  fwd_tables<N>(ra0, ra1, pm0, pm1, d0, d1, a.wc + (size_t)b * kWaveConsts);
   __syncthreads();
   float2* ck_seg = a.ckpt ? a.ckpt + (size_t)bm * K * NN : nullptr;
   float2* vh_seg = a.vhat ? a.vhat + (size_t)bm * K * NN : nullptr;
@@ -1141,10 +1194,10 @@ __device__ __forceinline__ int adj_wave(int w, int waves, int MK) {
 }
 
 struct AdjArgs {
-  int M, Ko, Nz, H, W, Ntot, global_tilt, grad_mask;  // Ko: object modes
-  float dx, lam;
+  int M, Ko, Nz, H, W, Ntot, grad_mask;  // Ko: object modes
   const int32_t* idx;
-  const float *pos, *tilt, *dz;
+  const float* pos;
+  const Pair* wc;  // [batch entry][kWaveConsts]
   const float2* T;
   const float2* Phat;
   // entering wave of slice s at ckpt[wave][s - ck_first], spectrum entering slice s at
@@ -1396,10 +1449,8 @@ __global__ void __launch_bounds__(T, Launch<N>::MINB_A) k_adjoint(AdjArgs a) {
   const int b = bm / (a.M * Ko), m = (bm / Ko) % a.M;  // waves: (position, probe mode, object mode)
   const int j = checked_index(a.idx, b, a.Ntot, a.status);
   int i0, i1;
-  float d0, d1, th0, th1;
+  float d0, d1;
   patch_corner<N>(a.pos, j, a.H, a.W, &i0, &i1, &d0, &d1, a.status);
-  tilt_of(a.tilt, a.global_tilt, j, &th0, &th1);
-  const float dz = a.dz[0];
   const bool want_obj = (a.grad_mask & (PTY_GRAD_AMP | PTY_GRAD_PHASE)) != 0;
   const bool want_probe = (a.grad_mask & PTY_GRAD_PROBE) != 0;
   const bool want_pos = (a.grad_mask & PTY_GRAD_POS) != 0;
@@ -1470,7 +1521,7 @@ __global__ void __launch_bounds__(T, Launch<N>::MINB_A) k_adjoint(AdjArgs a) {
   }
 
   build_twiddles<N>(tw);
-  adj_tables<N>(cm0, cm1, cr0, cr1, e0, e1, c0, c1, f0, f1, d0, d1, th0, th1, dz, a.dx, a.lam);
+  adj_tables<N>(cm0, cm1, cr0, cr1, e0, e1, c0, c1, f0, f1, d0, d1, a.wc + (size_t)b * kWaveConsts);
 #if PTY_ADJ_L1PF
   if (want_obj) prefetch_l1(ck_base + (size_t)(a.s1 - 1) * NN, PTY_ADJ_L1PF * 1024);
 #endif
@@ -1925,13 +1976,9 @@ struct Pass {
     fa.H = pb.H;
     fa.W = pb.W;
     fa.Ntot = pb.Ntot;
-    fa.global_tilt = pb.global_tilt;
-    fa.dx = pb.dx;
-    fa.lam = pb.lam;
     fa.idx = pb.idx;
     fa.pos = pb.pos;
-    fa.tilt = pb.tilt;
-    fa.dz = pb.dz;
+    fa.wc = ws.wc;
     fa.T = ws.T;
     fa.Phat = ws.Phat;
     fa.ckpt = nullptr;
@@ -1948,10 +1995,25 @@ struct Pass {
 
   // T and probe spectra (start of every forward).
   int forward_begin() {
-    const size_t nobj = (size_t)pb.Ko * pb.Nz * pb.H * pb.W;
     prof_begin(st);
-    k_prepare_object<<<object_blocks(), 256, 0, st>>>(pb.amp, pb.phase, ws.T, nullptr, nobj);
-    PTY_LAUNCH_CHECK("k_prepare_object", 0);
+    PrepArgs pa;
+    pa.amp = pb.amp;
+    pa.phase = pb.phase;
+    pa.T = ws.T;
+    pa.n = (size_t)pb.Ko * pb.Nz * pb.H * pb.W;
+    pa.blocks = (int)object_blocks();
+    pa.B = pb.B;
+    pa.Ntot = pb.Ntot;
+    pa.global_tilt = pb.global_tilt;
+    pa.lam = pb.lam;
+    pa.kq = 1.0 / (N * (double)pb.dx);
+    pa.idx = pb.idx;
+    pa.tilt = pb.tilt;
+    pa.dz = pb.dz;
+    pa.wc = ws.wc;
+    pa.status = ws.status;
+    k_prepare<<<pa.blocks + (pb.B + 63) / 64, 256, 0, st>>>(pa);
+    PTY_LAUNCH_CHECK("k_prepare", 0);
     PTY_LAUNCH_RC(launch_waves<C>(k_probe_spectrum<N, T>, pb.M, T, probe_smem(), st, pb.probe, ws.Phat,
                                    (float2*)nullptr),
                   "k_probe_spectrum", 1);
@@ -2063,14 +2125,10 @@ struct Pass {
     aa.H = pb.H;
     aa.W = pb.W;
     aa.Ntot = pb.Ntot;
-    aa.global_tilt = pb.global_tilt;
     aa.grad_mask = pb.grad_mask;
-    aa.dx = pb.dx;
-    aa.lam = pb.lam;
     aa.idx = pb.idx;
     aa.pos = pb.pos;
-    aa.tilt = pb.tilt;
-    aa.dz = pb.dz;
+    aa.wc = ws.wc;
     aa.T = ws.T;
     aa.Phat = ws.Phat;
     aa.Psi = ws.Psi;

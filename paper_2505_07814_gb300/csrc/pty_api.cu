@@ -83,6 +83,7 @@ size_t layout_workspace(const pty_geom& g, int B, int mode, char* base, Workspac
   };
   w.status = (int*)take(sizeof(int) * 64);
   w.scal = (double*)take(sizeof(double) * 4);
+  w.wc = (Pair*)take(sizeof(float) * kWaveConstFloats * (size_t)(B > 0 ? B : 1));
   w.T = (float2*)take(sizeof(float2) * nobj);
   w.Phat = (float2*)take(sizeof(float2) * g.M * NN);
   w.Imode = (float*)take(sizeof(float) * waves * NN);
@@ -553,8 +554,12 @@ int pty_supported_sizes(void) { return (1 << 6) | (1 << 7) | (1 << 8); }
 
 namespace {
 constexpr size_t kNoallocBytes = (size_t)PTY_NOALLOC_SCRATCH_BYTES;
+// Room on top for the batch entries' table constants, which do not count against the documented limit: a
+// pattern's intensities alone take 4 * 64^2 bytes, so a batch under it has at most 2048 entries.
+size_t wave_const_bytes(int B) { return align_up(sizeof(float) * kWaveConstFloats * (size_t)(B > 0 ? B : 1)); }
+constexpr size_t kNoallocExtra = sizeof(float) * kWaveConstFloats * 2048 + 256;
 // Loaded with the library's device code on every GPU that uses it and held until the process exits.
-__device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocBytes];
+__device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocBytes + kNoallocExtra];
 // Device address of g_noalloc_scratch per device ordinal (host code may not use the symbol itself).
 // Filled without a lock: two host threads making their first call on a device at once both look
 // the address up and store the same value, which is harmless.  cudaDeviceReset would make a cached
@@ -572,9 +577,9 @@ int pty_loss_grad_noalloc(const pty_geom* geom, int B, const int32_t* idx, const
   int rc = validate_geom(geom);
   if (rc) return rc;
   REQUIRE(B >= 0, "batch size %d < 0", B);
-  const size_t need = layout_workspace(*geom, B, MODE_GRAD, nullptr, nullptr);
+  const size_t need = layout_workspace(*geom, B, MODE_GRAD, nullptr, nullptr) - wave_const_bytes(B);
   if (need > kNoallocBytes) {
-    const size_t empty = layout_workspace(*geom, 0, MODE_GRAD, nullptr, nullptr);
+    const size_t empty = layout_workspace(*geom, 0, MODE_GRAD, nullptr, nullptr) - wave_const_bytes(0);
     if (empty > kNoallocBytes)
       set_error("pty_loss_grad_noalloc: the object alone needs %zu bytes of scratch (transmission and its "
                 "gradient) but the fixed area holds %zu; no batch fits; use pty_loss_grad with a caller-owned "
@@ -600,7 +605,7 @@ int pty_loss_grad_noalloc(const pty_geom* geom, int B, const int32_t* idx, const
   }
   void* ws = g_noalloc_addr[dev];
   rc = pty_loss_grad(geom, B, idx, amp, phase, probe, pos, tilt, dz, I_meas, loss, I_model, g_amp, g_phase, g_probe,
-                     g_pos, g_tilt, g_dz, accumulate, ws, kNoallocBytes, stream);
+                     g_pos, g_tilt, g_dz, accumulate, ws, kNoallocBytes + kNoallocExtra, stream);
   if (rc == PTY_OK && status) {
     if (cudaMemcpyAsync(status, ws, sizeof(int), cudaMemcpyDeviceToDevice, (cudaStream_t)stream) != cudaSuccess) {
       set_error("pty_loss_grad_noalloc: status copy failed: %s", cudaGetErrorString(cudaGetLastError()));

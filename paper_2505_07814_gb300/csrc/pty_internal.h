@@ -10,8 +10,11 @@ namespace pty {
 
 // Workspace carve-up (all pieces 256-byte aligned).  k-space arrays use the FFT's digit-ordered
 // layout: element p1 * N + p0 holds frequency (kbin(p0), kbin(p1)) along (axis 0, axis 1).
+struct Pair;       // pipeline.cuh
+constexpr int kWaveConstFloats = 16;
 struct Workspace {
   int* status;     // [1]   device status bits
+  Pair* wc;        // [B][8] pairs of floats: constants of each batch entry's propagator tables
   float2* T;       // [Ko][Nz][H][W]  transmission amp * exp(i phase)
   float2* Phat;    // [M][N*N]        probe spectra F[P_m] (k-space layout)
   float2* ckpt;     // [B][M][Nz][N*N] wave entering each slice (natural layout); recompute mode:
