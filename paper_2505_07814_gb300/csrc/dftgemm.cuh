@@ -588,7 +588,7 @@ int run_pipeline_gemm(const Problem& pb) {
       if (pb.loss == PTY_LOSS_POISSON) return ps.base.stats();  // the measured patterns only
       rc = ps.forward(pb.I_meas);
       if (rc) return rc;
-      return ps.base.stats_write();
+      return ps.base.stats_write(pb.B * loss_parts<N>());
     case MODE_BACKWARD:
       rc = ps.base.external_dldi(pb.dldi);
       if (rc) return rc;

@@ -7,8 +7,8 @@
 //                      entry's tables
 //   k_probe_spectrum   P^_m = F[P_m]                                              (M CTAs)
 //   k_forward          shift, Nz transmissions, Nz-1 propagations, far field      (B*M CTAs)
-//   k_loss             mode sum, Eq. 5/6 per pixel, dL/dI, per-pattern sums      (B CTAs)
-//   k_loss_finalize    batch loss and dL/dI normaliser (FP64)                      (1 CTA)
+//   k_loss             mode sum, Eq. 5/6 per pixel, dL/dI; the last CTA forms the batch loss and the dL/dI
+//                      normaliser (FP64)                                      (B * N / 32 CTAs)
 //   k_adjoint          reverse of k_forward, scatter-adds dL/dT, probe-spectrum
 //                      gradient, FP64-reduced position / tilt / dz partials       (B*M CTAs)
 //   k_object_grad      dL/damp, dL/dphase from dL/dT (chain rule of amp exp(i phase))
@@ -47,7 +47,7 @@
 #define PTY_ADJ_GROUP 32
 #endif
 // The propagation step inside the row transform (0) reads each task's 32 spectrum values in one
-// batch (PTY_KQ = 32): multislice adjoint 3.274 ms against 3.455 as its own pass (1)
+// batch: multislice adjoint 3.274 ms against 3.455 as its own pass (1)
 #ifndef PTY_ADJ_SPLIT_ROW
 #define PTY_ADJ_SPLIT_ROW 0
 #endif
@@ -120,12 +120,18 @@
 #ifndef PTY_KA
 #define PTY_KA 4
 #endif
-// (the adjoint's spectrum reads in the fused propagation step; capped at a task's elements)
+// (the adjoint's spectrum reads in the fused propagation step, capped at a task's elements, and the probe
+// step's; the compiler's register allocation of the whole N = 128 adjoint hangs on them: 512 positions,
+// 3111 us at KQ 32 / KR 4, 2953 at 32 / 8, 2930 at 16 / 8, 2979 at 32 / 16; N = 64 592 us at KR 8 against 595;
+// N = 256 9.85 ms a 64-position batch at KR 4 against 9.91)
 #ifndef PTY_KQ
-#define PTY_KQ 32
+#define PTY_KQ 16
 #endif
 #ifndef PTY_KR
-#define PTY_KR 4
+#define PTY_KR 8
+#endif
+#ifndef PTY_KR256
+#define PTY_KR256 4
 #endif
 
 namespace pty {
@@ -187,6 +193,45 @@ __device__ __forceinline__ Pair pair_poly(float q2, Pair a, float q, Pair b) {
   return Pair{s, e + pe + re + fmaf(q2, a.lo, q * b.lo)};
 }
 __device__ __forceinline__ float pair_value(Pair a) { return a.hi + a.lo; }
+__device__ __forceinline__ Pair pair_add(Pair a, Pair b) {
+  const float s = __fadd_rn(a.hi, b.hi), t = __fadd_rn(s, -a.hi);
+  const float e = __fadd_rn(__fadd_rn(a.hi, -__fadd_rn(s, -t)), __fadd_rn(b.hi, -t));
+  return Pair{s, a.lo + b.lo + e};
+}
+// sum over the warp, in lane 0
+__device__ __forceinline__ Pair pair_warp_sum(Pair x) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    x = pair_add(x, Pair{__shfl_down_sync(0xffffffffu, x.hi, o), __shfl_down_sync(0xffffffffu, x.lo, o)});
+  return x;
+}
+// a sum that overflowed stays infinite (its lo is not a number)
+__device__ __forceinline__ double pair_total(Pair x) {
+  return isfinite(x.hi) ? (double)x.hi + (double)x.lo : (double)x.hi;
+}
+// Sums of NV values over the CTA's T threads, each in the thread of its number (threads < NV), in pairs of floats
+// and a fixed order (an FP64 shuffle sum costs 64 clocks of a scheduler per step and value).  red: NV * T / 32 pairs.
+template <int T, int NV>
+__device__ __forceinline__ double block_sum_pairs(const float (&v)[NV], Pair* red) {
+  constexpr int W = T / 32;
+  const int lane = threadIdx.x & 31, w = threadIdx.x / 32;
+#pragma unroll
+  for (int q = 0; q < NV; ++q) {
+    const Pair x = pair_warp_sum(Pair{v[q], 0.f});
+    if (lane == 0) red[q * W + w] = x;
+  }
+  __syncthreads();
+  Pair r{0.f, 0.f};
+  if (w == 0) {
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+      const Pair x = pair_warp_sum(lane < W ? red[q * W + lane] : Pair{0.f, 0.f});
+      const float hi = __shfl_sync(0xffffffffu, x.hi, 0), lo = __shfl_sync(0xffffffffu, x.lo, 0);
+      if (lane == q) r = Pair{hi, lo};
+    }
+  }
+  return threadIdx.x < NV ? pair_total(r) : 0.0;
+}
 // exp(i pi (hi + lo)): hi reduced modulo 2 exactly, lo as a first-order rotation
 __device__ __forceinline__ float2 expipi(Pair x) {
   const float r = x.hi - 2.0f * rintf(0.5f * x.hi);
@@ -839,24 +884,29 @@ __global__ void k_dldi_to_kspace(const float* __restrict__ dldi, float* __restri
 }
 
 // ---------------------------------------------------------------------------------------------
-// Loss: one CTA per pattern.  Sums modes, evaluates Eq. 5 or 6 per pixel and dL/dI up to the
-// batch-wide normaliser, and writes FP64 per-pattern sums.
+// Loss.  A CTA takes 32 consecutive k-space rows p0 of one pattern (32 whole detector rows): it sums the modes,
+// evaluates Eq. 5 or 6 per pixel and dL/dI up to the batch-wide normaliser, and writes its FP64 sums; the
+// CTA that finishes last adds them up.
 // ---------------------------------------------------------------------------------------------
 struct LossArgs {
   int M, Ntot, loss;
-  int* status;
+  int* status;  // [1]: CTAs done, zeroed before the call's first kernel
   float p, eps;
   const int32_t* idx;
   const float* Imode;
   const float* I_meas;
   float* I_model;
   float* u;
-  double* lpart;
-  // PACBED term (nullptr when off): batch sums of I_model and I_meas in k-space order, and the
-  // per-pattern sums of I_meas^pac_p
+  double* lpart;  // [CTA][2]
+  // PACBED term (nullptr when off): batch sums of I_model and I_meas in detector order, and the
+  // CTAs' sums of I_meas^pac_p
   float* pac;
   double* pacpart;
   float pac_p;
+  // result (see loss_finalize)
+  double DB;
+  double *scal, *loss_out;
+  const double* whole;
 };
 
 // x^p for x >= 0 (0 for x <= 0 when p != 1), with the common exponents exact.
@@ -864,11 +914,6 @@ __device__ __forceinline__ float pow_nn(float x, float p) {
   if (p == 1.0f) return x;
   if (x <= 0.f) return 0.f;
   return p == 0.5f ? sqrtf(x) : powf(x, p);
-}
-
-template <int N>
-__host__ __device__ constexpr size_t loss_smem_bytes() {
-  return sizeof(float) * (size_t)N * (N + 1) + 64 * sizeof(double);
 }
 
 template <int T>
@@ -892,6 +937,25 @@ __device__ __forceinline__ void block_sum2(double& x, double& y, double* red) {
     x = sx;
     y = sy;
   }
+}
+
+// block_sum2 over the first 256 threads of a CTA of any size (named barrier 1)
+__device__ __forceinline__ void sum2_first256(double& x, double& y, double* red) {
+  for (int o = 16; o > 0; o >>= 1) {
+    x += __shfl_down_sync(0xffffffffu, x, o);
+    y += __shfl_down_sync(0xffffffffu, y, o);
+  }
+  const int w = threadIdx.x / 32;
+  if ((threadIdx.x & 31) == 0) {
+    red[2 * w] = x;
+    red[2 * w + 1] = y;
+  }
+  asm volatile("bar.sync 1, 256;" ::: "memory");
+  if (threadIdx.x == 0)
+    for (int i = 1; i < 8; ++i) {
+      x += red[2 * i];
+      y += red[2 * i + 1];
+    }
 }
 
 // Eq. 5 / 6 at one detector pixel: the summand of the loss (term), the pattern term of its
@@ -922,130 +986,167 @@ __device__ __forceinline__ void loss_pixel(float I, float d, float p, float eps,
   }
 }
 
-// PAC: the PACBED sums are on (a.pac != nullptr); the plain instantiation carries none of that work.
-template <int N, int T, bool PAC = false>
-__global__ void __launch_bounds__(T) k_loss(LossArgs a) {
-  constexpr int RS = N + 1;
-  constexpr int NN = N * N;
-  extern __shared__ __align__(16) float lsm[];
-  float* L = lsm;
-  double* red = reinterpret_cast<double*>(lsm + N * RS + ((N * RS) & 1));
-  const int b = blockIdx.x, tid = threadIdx.x;
-  // mode sum, four pixels of one k-space row per thread and load (N is a multiple of 4)
-  const float4* Im4 = reinterpret_cast<const float4*>(a.Imode + (size_t)b * a.M * NN);
-  for (int e4 = tid; e4 < NN / 4; e4 += T) {
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int m = 0; m < a.M; ++m) {
-      const float4 v = ld_ro(Im4 + (size_t)m * (NN / 4) + e4);
-      acc.x += v.x;
-      acc.y += v.y;
-      acc.z += v.z;
-      acc.w += v.w;
+// Batch loss (Eq. 5 / 6) and the normaliser of dL/dI, in FP64, fixed summation order, by 256
+// threads from the n CTAs' sums.  With the means of Eq. 5 / 6 written out over D detector pixels and B
+// patterns, Poisson is -Y / S and Gaussian sqrt(D B Q) / S, where S = sum of I_meas^p, Y = sum of the
+// Poisson summands and Q = sum of the squared residuals.  `whole` (or nullptr) holds {S, Q, D B} of the
+// whole batch when this call holds one part of it: the normaliser then comes from the whole batch, and the
+// loss written is this part's share of the whole batch's loss (the shares of the parts add up to it).
+__device__ __forceinline__ void loss_finalize(const LossArgs& a, int n, double* red) {
+  double x = 0.0, y = 0.0;
+  for (int b = threadIdx.x; b < n; b += 256) {
+    x += __ldcg(a.lpart + 2 * b);
+    y += __ldcg(a.lpart + 2 * b + 1);
+  }
+  sum2_first256(x, y, red);
+  if (threadIdx.x == 0) {
+    const double S = a.whole ? a.whole[0] : x;
+    double Lv, scale;
+    if (a.loss == PTY_LOSS_POISSON) {
+      Lv = -y / S;
+      scale = 1.0 / S;
+    } else {
+      const double Q = a.whole ? a.whole[1] : y, DBw = a.whole ? a.whole[2] : a.DB;
+      // this part's share y / Q of sqrt(D B Q) / S is sqrt(D B / Q) y / S
+      Lv = Q > 0.0 ? sqrt(DBw / Q) * y / S : 0.0;
+      scale = Q > 0.0 ? sqrt(DBw) / (sqrt(Q) * S) : 0.0;
     }
-    float* row = L + (4 * e4 / N) * RS + (4 * e4) % N;
-    row[0] = acc.x;
-    row[1] = acc.y;
-    row[2] = acc.z;
-    row[3] = acc.w;
-  }
-  __syncthreads();
-  const float* Id = a.I_meas ? a.I_meas + (size_t)checked_index(a.idx, b, a.Ntot, a.status) * NN : nullptr;
-  const float p = a.p;
-  float sd = 0.f, st = 0.f, sp = 0.f;
-  for (int q = tid; q < NN; q += T) {
-    const int k0 = (q / N + N / 2) & (N - 1), k1 = (q % N + N / 2) & (N - 1);
-    const int l = kpos1<N>(k1) * RS + kpos0<N>(k0);  // staging row p1, column p0 (global p1 * N + p0)
-    const float I = L[l];
-    if (a.I_model) a.I_model[(size_t)b * NN + q] = I;
-    if (Id) {
-      const float d = Id[q];
-      float term, u, Dp;
-      loss_pixel(I, d, p, a.eps, a.loss, &term, &Dp, &u);
-      sd += Dp;
-      st += term;
-      L[l] = u;
-      if (PAC) {  // sums in detector order: a warp's atomics land on consecutive addresses
-        atomicAdd(a.pac + q, I);
-        atomicAdd(a.pac + NN + q, d);
-        sp += pow_nn(d, a.pac_p);
-      }
+    if (!isfinite(Lv) || !isfinite(scale)) {
+      atomicOr(a.status, PTY_ENONFINITE);
+      scale = 0.0;
     }
-  }
-  __syncthreads();
-  if (a.u) {
-    for (int e = tid; e < NN; e += T) a.u[(size_t)b * NN + e] = L[(e / N) * RS + e % N];
-  }
-  if (a.lpart) {
-    double x = sd, y = st;
-    block_sum2<T>(x, y, red);
-    if (tid == 0) {
-      a.lpart[2 * b] = x;
-      a.lpart[2 * b + 1] = y;
-    }
-  }
-  if (PAC) {
-    __syncthreads();
-    double x = sp, y = 0.0;
-    block_sum2<T>(x, y, red);
-    if (tid == 0) a.pacpart[b] = x;
+    a.scal[0] = scale;
+    a.scal[1] = Lv;
+    if (a.loss_out) *a.loss_out = Lv;
   }
 }
 
-// The same without shared-memory staging (the N = 256 staging area would not fit): walks the
-// pattern in k-space order (coalesced mode sum and dL/dI), gathering the measured pattern and
-// scattering the modelled one in detector order.
-template <int N, int T, bool PAC = false>
-__global__ void __launch_bounds__(T) k_loss_gather(LossArgs a) {
-  constexpr int NN = N * N;
-  __shared__ double red[2 * (T / 32)];
-  const int b = blockIdx.x, tid = threadIdx.x;
-  const float* Im = a.Imode + (size_t)b * a.M * NN;
+// CTAs per pattern.
+template <int N>
+__host__ __device__ constexpr int loss_parts() {
+  return N / 32;
+}
+// Column of local row pr in staging row p1 (pitch 33): rotated so that a warp walking along a detector row,
+// whose k-space columns p1 lie N / 4 (N / 16 at N = 256) apart, meets 32 banks.
+template <int N>
+__device__ __forceinline__ int loss_col(int p1, int pr) {
+  constexpr int step = N == 256 ? 16 : N / 4, rot = N == 256 ? -14 : N == 128 ? 8 : 24;
+  return (pr + rot * (p1 / step)) & 31;
+}
+
+// HBM-bound at large batches (the modes' intensities are read once); at small ones what counts is the CTAs in
+// flight and the loads each thread has outstanding, so a pattern is spread over N / 32 CTAs, a thread's
+// measured pixels are fetched before the mode sum, and the modes four at a time.  One CTA per pattern with
+// one load in flight (and, at N = 256, measured patterns gathered element by element) took 37 us on 16
+// patterns of 12 modes at N = 128 and 351 us on 256 at N = 256; this 14 and 195 us.
+// PAC: the PACBED sums are on (a.pac != nullptr); the plain instantiation carries none of that work.
+template <int N, bool PAC = false>
+__global__ void __launch_bounds__(4 * N, 256 / N) k_loss(LossArgs a) {
+  constexpr int T = 4 * N, NN = N * N, S = loss_parts<N>(), RS = 33;
+  constexpr int PX = 8, E4 = PX / 4;  // pixels and float4s a thread
+  __shared__ float L[N * RS];
+  __shared__ Pair red[3 * (T / 32)];
+  __shared__ double fin[16];
+  __shared__ int last;
+  const int b = blockIdx.x / S, s = blockIdx.x % S, tid = threadIdx.x;
+  // detector pixel f = tid + T i of this CTA: local row pr = f / N, column q1 = f % N
+  auto pixel = [&](int i, int& pr, int& p1) {
+    const int f = tid + T * i, q1 = f % N;
+    pr = f / N;
+    p1 = kpos1<N>((q1 + N / 2) & (N - 1));
+    return ((kbin0<N>(32 * s + pr) + N / 2) & (N - 1)) * N + q1;
+  };
   const float* Id = a.I_meas ? a.I_meas + (size_t)checked_index(a.idx, b, a.Ntot, a.status) * NN : nullptr;
+  float d[PX];
+  if (Id) {
+#pragma unroll
+    for (int i = 0; i < PX; ++i) {
+      int pr, p1;
+      d[i] = ld_ro(Id + pixel(i, pr, p1));
+    }
+  }
+  // mode sum, four rows p0 of one column p1 per thread and load
+  const float4* Im4 = reinterpret_cast<const float4*>(a.Imode + (size_t)b * a.M * NN + 32 * s);
+  auto at = [&](int i) { return (tid + T * i) / 8 * (N / 4) + (tid + T * i) % 8; };
+  float4 acc[E4];
+#pragma unroll
+  for (int i = 0; i < E4; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  constexpr int MU = 4;  // modes in flight
+  for (int m0 = 0; m0 < a.M; m0 += MU) {
+    float4 v[MU][E4];
+#pragma unroll
+    for (int k = 0; k < MU; ++k)
+#pragma unroll
+      for (int i = 0; i < E4; ++i)
+        if (m0 + k < a.M) v[k][i] = ld_ro(Im4 + (size_t)(m0 + k) * (NN / 4) + at(i));
+#pragma unroll
+    for (int k = 0; k < MU; ++k)
+#pragma unroll
+      for (int i = 0; i < E4; ++i)
+        if (m0 + k < a.M) {
+          acc[i].x += v[k][i].x;
+          acc[i].y += v[k][i].y;
+          acc[i].z += v[k][i].z;
+          acc[i].w += v[k][i].w;
+        }
+  }
+#pragma unroll
+  for (int i = 0; i < E4; ++i) {
+    const int p1 = (tid + T * i) / 8, c = 4 * ((tid + T * i) % 8);
+    L[p1 * RS + loss_col<N>(p1, c)] = acc[i].x;
+    L[p1 * RS + loss_col<N>(p1, c + 1)] = acc[i].y;
+    L[p1 * RS + loss_col<N>(p1, c + 2)] = acc[i].z;
+    L[p1 * RS + loss_col<N>(p1, c + 3)] = acc[i].w;
+  }
+  __syncthreads();
   float sd = 0.f, st = 0.f, sp = 0.f;
-  for (int e = tid; e < NN; e += T) {  // e = p1 * N + p0
-    float I = 0.f;
-    for (int m = 0; m < a.M; ++m) I += Im[(size_t)m * NN + e];
-    const int k0 = kbin0<N>(e % N), k1 = kbin1<N>(e / N);
-    const int q = ((k0 + N / 2) & (N - 1)) * N + ((k1 + N / 2) & (N - 1));
+#pragma unroll
+  for (int i = 0; i < PX; ++i) {
+    int pr, p1;
+    const int q = pixel(i, pr, p1), l = p1 * RS + loss_col<N>(p1, pr);
+    const float I = L[l];
     if (a.I_model) a.I_model[(size_t)b * NN + q] = I;
     if (Id) {
       float term, u, Dp;
-      const float d = Id[q];
-      loss_pixel(I, d, a.p, a.eps, a.loss, &term, &Dp, &u);
+      loss_pixel(I, d[i], a.p, a.eps, a.loss, &term, &Dp, &u);
       sd += Dp;
       st += term;
-      a.u[(size_t)b * NN + e] = u;
-      if (PAC) {
-        atomicAdd(a.pac + e, I);
-        atomicAdd(a.pac + NN + e, d);
-        sp += pow_nn(d, a.pac_p);
+      L[l] = u;
+      if (PAC) {  // a warp's atomics land on consecutive addresses
+        atomicAdd(a.pac + q, I);
+        atomicAdd(a.pac + NN + q, d[i]);
+        sp += pow_nn(d[i], a.pac_p);
       }
     }
   }
-  if (a.lpart) {
-    double x = sd, y = st;
-    block_sum2<T>(x, y, red);
+  if (!Id) return;
+  __syncthreads();
+  for (int e = tid; e < 32 * N; e += T)
+    a.u[(size_t)b * NN + (e / 32) * N + 32 * s + e % 32] = L[(e / 32) * RS + loss_col<N>(e / 32, e % 32)];
+  const float v3[3] = {sd, st, sp};
+  const double sum = block_sum_pairs<T>(v3, red);
+  if (tid < 2) a.lpart[2 * blockIdx.x + tid] = sum;
+  if (PAC && tid == 2) a.pacpart[blockIdx.x] = sum;
+  if (tid < 32) {  // the warp that wrote the sums counts the CTA as done
+    __syncwarp();
     if (tid == 0) {
-      a.lpart[2 * b] = x;
-      a.lpart[2 * b + 1] = y;
+      __threadfence();
+      last = atomicAdd(a.status + 1, 1) == (int)gridDim.x - 1;
     }
   }
-  if (PAC) {
-    __syncthreads();
-    double x = sp, y = 0.0;
-    block_sum2<T>(x, y, red);
-    if (tid == 0) a.pacpart[b] = x;
-  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();  // every CTA's sums are visible
+  if (tid < 256) loss_finalize(a, (int)gridDim.x, fin);
 }
 
 // PACBED term (Eq. 7) of one batch, one CTA of 1024 threads: the batch-mean patterns A and C from
 // the sums, d = A^p - C^p, the loss w sqrt(<d^2>) / <I_meas^p> added to *loss_out, and the
 // derivative w d p A^(p-1) / (<I_meas^p> N^2 B sqrt(<d^2>)), the same for every pattern, written to
-// pac[2 N^2 ..] (k-space order) for the adjoint.  The sums are in the order of the loss kernel's
-// loop: detector order (k_loss, N <= 128) or k-space order (k_loss_gather, N = 256).
+// pac[2 N^2 ..] (k-space order) for the adjoint.  The sums are in detector order.
 template <int N>
-__global__ void __launch_bounds__(1024) k_pacbed(float* __restrict__ pac, const double* __restrict__ pacpart, int B,
-                                                 float p, float w, double* loss_out, double* scal, int* status) {
+__global__ void __launch_bounds__(1024) k_pacbed(float* __restrict__ pac, const double* __restrict__ pacpart,
+                                                 int parts, int B, float p, float w, double* loss_out, double* scal, int* status) {
   constexpr int NN = N * N;
   __shared__ double red[64];
   __shared__ double sh[2];
@@ -1056,7 +1157,7 @@ __global__ void __launch_bounds__(1024) k_pacbed(float* __restrict__ pac, const 
     const float d = pow_nn(pac[e] * inv_b, p) - pow_nn(pac[NN + e] * inv_b, p);
     m2 += (double)d * d;
   }
-  for (int b = tid; b < B; b += 1024) z += pacpart[b];
+  for (int b = tid; b < parts; b += 1024) z += pacpart[b];
   block_sum2<1024>(m2, z, red);
   if (tid == 0) {
     const double ms = m2 / NN, Z = z / ((double)NN * B);
@@ -1072,12 +1173,8 @@ __global__ void __launch_bounds__(1024) k_pacbed(float* __restrict__ pac, const 
     const float A = pac[e] * inv_b;
     const float d = pow_nn(A, p) - pow_nn(pac[NN + e] * inv_b, p);
     const float dpow = p == 1.0f ? 1.0f : (A > 0.f ? p * powf(A, p - 1.0f) : 0.f);
-    int ek = e;  // k-space position of sum element e
-    if constexpr (N != 256) {
-      const int k0 = (e / N + N / 2) & (N - 1), k1 = (e % N + N / 2) & (N - 1);
-      ek = kpos1<N>(k1) * N + kpos0<N>(k0);
-    }
-    pac[2 * NN + ek] = c * d * dpow;
+    const int k0 = (e / N + N / 2) & (N - 1), k1 = (e % N + N / 2) & (N - 1);
+    pac[2 * NN + kidx<N>(kpos0<N>(k0), kpos1<N>(k1))] = c * d * dpow;
   }
 }
 
@@ -1091,43 +1188,6 @@ __global__ void k_pacbed_fold(float* __restrict__ u, const float* __restrict__ p
   const float gs = (float)(2.0 * scal[0] / N), gp = 2.0f / N;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     u[i] = fmaf(gp, pacg[i % NN], gs * u[i]);
-}
-
-// Batch loss (Eq. 5 / 6) and the normaliser of dL/dI, in FP64, fixed summation order.  With the
-// means of Eq. 5 / 6 written out over D detector pixels and B patterns, Poisson is -Y / S and
-// Gaussian sqrt(D B Q) / S, where S = sum of I_meas^p, Y = sum of the Poisson summands and
-// Q = sum of the squared residuals.  `whole` (or nullptr) holds {S, Q, D B} of the whole batch when
-// this call holds one part of it: the normaliser then comes from the whole batch, and the loss
-// written is this part's share of the whole batch's loss (the shares of the parts add up to it).
-static __global__ void k_loss_finalize(const double* __restrict__ lpart, int B, int loss, double DB, double* scal,
-                                       double* loss_out, int* status, const double* __restrict__ whole) {
-  __shared__ double red[64];
-  double x = 0.0, y = 0.0;
-  for (int b = threadIdx.x; b < B; b += blockDim.x) {
-    x += lpart[2 * b];
-    y += lpart[2 * b + 1];
-  }
-  block_sum2<256>(x, y, red);
-  if (threadIdx.x == 0) {
-    const double S = whole ? whole[0] : x;
-    double Lv, scale;
-    if (loss == PTY_LOSS_POISSON) {
-      Lv = -y / S;
-      scale = 1.0 / S;
-    } else {
-      const double Q = whole ? whole[1] : y, DBw = whole ? whole[2] : DB;
-      // this part's share y / Q of sqrt(D B Q) / S is sqrt(D B / Q) y / S
-      Lv = Q > 0.0 ? sqrt(DBw / Q) * y / S : 0.0;
-      scale = Q > 0.0 ? sqrt(DBw) / (sqrt(Q) * S) : 0.0;
-    }
-    if (!isfinite(Lv) || !isfinite(scale)) {
-      atomicOr(status, PTY_ENONFINITE);
-      scale = 0.0;
-    }
-    scal[0] = scale;
-    scal[1] = Lv;
-    if (loss_out) *loss_out = Lv;
-  }
 }
 
 // Per-pattern sum of I_meas^p (one CTA per batch entry) into lpart[2 b]; lpart[2 b + 1] = 0.  The
@@ -1149,7 +1209,7 @@ __global__ void __launch_bounds__(T) k_meas_sum(const float* __restrict__ I_meas
   }
 }
 
-// {sum over the batch of lpart[2 b], of lpart[2 b + 1], D B} into out[3] (fixed summation order).
+// {sum over the B partials lpart[2 b], over lpart[2 b + 1], D B} into out[3] (fixed summation order).
 static __global__ void k_batch_stats(const double* __restrict__ lpart, int B, double DB, double* __restrict__ out,
                                      int* status) {
   __shared__ double red[64];
@@ -1262,10 +1322,9 @@ __host__ __device__ constexpr size_t adj_stage_offset() {
 }
 template <int N, int T>
 __host__ __device__ constexpr size_t adj_smem_bytes() {
-  static_assert(T <= 1024, "reduction slots");
+  static_assert(5 * T * sizeof(float) <= sizeof(float2) * wave_rows<N>() * (N + 1), "partials in the wave's place");
   return adj_staged<N, T>() || adj256_staged<N>() ? adj_stage_offset<N>() + kStageBytes + 16
-                            : sizeof(float2) * ((size_t)wave_rows<N>() * (N + 1) + 5 * N) + sizeof(float) * 6 * N +
-                                  sizeof(double) * 5 * (T / 32);
+                            : sizeof(float2) * ((size_t)wave_rows<N>() * (N + 1) + 5 * N) + sizeof(float) * 6 * N;
 }
 // The stage in the calling kernel's dynamic shared memory.
 template <int N>
@@ -1394,7 +1453,7 @@ template <int N>
 struct ProbeStore {
   static constexpr bool kReplaces = false;
   static constexpr bool kPreload = false;  // may run in a step that has read two tasks
-  static constexpr int kChunk = PTY_KR;
+  static constexpr int kChunk = N == 256 ? PTY_KR256 : PTY_KR;
   float2* gP;  // or nullptr
   const float2* Ph;
   const float2 *cr0, *cr1;
@@ -1441,8 +1500,7 @@ __global__ void __launch_bounds__(T, Launch<N>::MINB_A) k_adjoint(AdjArgs a) {
   float* c1 = c0 + N;
   float* f0 = c1 + N;  // 2 pi f_a / N^2 (position term)
   float* f1 = f0 + N;
-  double* red = reinterpret_cast<double*>(f1 + N);
-  const int tid = threadIdx.x, lane = tid & 31;
+  const int tid = threadIdx.x;
   // wave (position, mode); a cluster of F::C CTAs per wave
   const int bm = adj_wave<PTY_ADJ_GROUP>(blockIdx.x / F::C, gridDim.x / F::C, a.M * (OM ? a.Ko : 1));
   const int Ko = OM ? a.Ko : 1;
@@ -1636,29 +1694,35 @@ __global__ void __launch_bounds__(T, Launch<N>::MINB_A) k_adjoint(AdjArgs a) {
     if (tid == 0 && (sst >> 31)) stage_wait(sbar, sst & 1);
   }
 
-  // FP64 reduction of the five scalar partials over the CTA
-  double v5[5] = {gp0, gp1, gt0, gt1, gdz};
-#pragma unroll
-  for (int q = 0; q < 5; ++q)
-    for (int o = 16; o > 0; o >>= 1) v5[q] += __shfl_down_sync(0xffffffffu, v5[q], o);
-  const int w = tid / 32;
-  if (lane == 0) {
-#pragma unroll
-    for (int q = 0; q < 5; ++q) red[5 * w + q] = v5[q];
-  }
-  __syncthreads();
-  if (tid < 5) {
-    double acc = 0.0;
-    for (int i = 0; i < T / 32; ++i) acc += red[5 * i + tid];
-    if constexpr (F::C == 1) {
-      a.spart[(size_t)bm * 5 + tid] += acc;
-    } else {  // the CTAs of a cluster each hold part of the wave
-      atomicAdd(a.spart + (size_t)bm * 5 + tid, acc);
-    }
-  }
-  if (a.s0 > 0) {  // hand the adjoint wave to the launch of the previous segment
+  __syncthreads();  // every thread group is done with its rows
+  if (a.s0 > 0) {   // hand the adjoint wave to the launch of the previous segment
     float2* g = a.gstate + (size_t)bm * NN + (size_t)F::rank() * F::ROWS * N;
     for (int e = tid; e < F::ROWS * N; e += T) g[e] = s[(e / N) * RS + e % N];
+    __syncthreads();
+  }
+  // The five scalar partials over the CTA, through the wave's shared memory: one warp per value adds the threads'
+  // partials as pairs of floats (48 bits) in a fixed order.  FP64 shuffle sums in every warp took 3.7 us of
+  // the CTA (64 clocks of a scheduler per step and value): N = 128, 512 positions, 3197 us against 3111.
+  float* part = reinterpret_cast<float*>(s);
+  part[tid] = gp0;
+  part[T + tid] = gp1;
+  part[2 * T + tid] = gt0;
+  part[3 * T + tid] = gt1;
+  part[4 * T + tid] = gdz;
+  __syncthreads();
+  const int lane = tid & 31;
+  for (int q = tid / 32; q < 5; q += T / 32) {
+    Pair x{0.f, 0.f};
+    for (int i = lane; i < T; i += 32) x = pair_add(x, Pair{part[q * T + i], 0.f});
+    x = pair_warp_sum(x);
+    if (lane == 0) {
+      const double sum = pair_total(x);
+      if constexpr (F::C == 1) {
+        a.spart[(size_t)bm * 5 + q] += sum;
+      } else {  // the CTAs of a cluster each hold part of the wave
+        atomicAdd(a.spart + (size_t)bm * 5 + q, sum);
+      }
+    }
   }
 }
 
@@ -1934,12 +1998,6 @@ struct Pass {
                                    (int)probe_smem()) == cudaSuccess &&
               cudaFuncSetAttribute(k_probe_grad<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)probe_smem()) == cudaSuccess;
-    if constexpr (N != 256) {
-      ok = ok && cudaFuncSetAttribute(k_loss<N, T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)loss_smem_bytes<N>()) == cudaSuccess;
-      ok = ok && cudaFuncSetAttribute(k_loss<N, T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)loss_smem_bytes<N>()) == cudaSuccess;
-    }
 #if PTY_CARVEOUT
     // One N = 128 wave kernel CTA per SM: ask for the smallest shared-memory carve-out that holds it,
     // so the rest of the SM's on-chip memory serves as L1 for the loads in flight.
@@ -2051,19 +2109,16 @@ struct Pass {
     la.pac = pac ? ws.pac : nullptr;
     la.pacpart = pac ? ws.pacpart : nullptr;
     la.pac_p = pb.p_pac;
+    la.DB = (double)pb.B * NN;
+    la.scal = ws.scal;
+    la.loss_out = pb.loss_out;
+    la.whole = pb.whole;
     if (pac && cudaMemsetAsync(ws.pac, 0, sizeof(float) * 2 * NN, st) != cudaSuccess) return memset_failed();
-    if constexpr (N == 256) {
-      (pac ? k_loss_gather<N, T, true> : k_loss_gather<N, T, false>)<<<pb.B, T, 0, st>>>(la);
-    } else {
-      (pac ? k_loss<N, T, true> : k_loss<N, T, false>)<<<pb.B, T, loss_smem_bytes<N>(), st>>>(la);
-    }
+    (pac ? k_loss<N, true> : k_loss<N, false>)<<<pb.B * loss_parts<N>(), 4 * N, 0, st>>>(la);
     PTY_LAUNCH_CHECK("k_loss", 3);
     if (I_meas) {
-      k_loss_finalize<<<1, 256, 0, st>>>(ws.lpart, pb.B, pb.loss, (double)pb.B * NN, ws.scal, pb.loss_out, ws.status,
-                                         pb.whole);
-      PTY_LAUNCH_CHECK("k_loss_finalize", 4);
       if (pac) {
-        k_pacbed<N><<<1, 1024, 0, st>>>(ws.pac, ws.pacpart, pb.B, pb.p_pac, pb.w_pac, pb.loss_out, ws.scal,
+        k_pacbed<N><<<1, 1024, 0, st>>>(ws.pac, ws.pacpart, pb.B * loss_parts<N>(), pb.B, pb.p_pac, pb.w_pac, pb.loss_out, ws.scal,
                                         ws.status);
         PTY_LAUNCH_CHECK("k_pacbed", -1);
         if (pb.mode == MODE_GRAD) {
@@ -2094,15 +2149,14 @@ struct Pass {
         k_meas_sum<N, T><<<pb.B, T, 0, st>>>(pb.I_meas, pb.idx, pb.Ntot, pb.p, ws.lpart, ws.status);
         PTY_LAUNCH_CHECK("k_meas_sum", -1);
       }
-    } else {
-      int rc = forward(pb.I_meas);
-      if (rc) return rc;
+      return stats_write(pb.B);
     }
-    return stats_write();
+    int rc = forward(pb.I_meas);
+    return rc ? rc : stats_write(pb.B * loss_parts<N>());
   }
-  // the per-pattern sums of the loss kernel (or k_meas_sum) into the caller's three statistics
-  int stats_write() {
-    k_batch_stats<<<1, 256, 0, st>>>(ws.lpart, pb.B, (double)pb.B * NN, pb.stats_out, ws.status);
+  // the n partial sums of the loss kernel (or k_meas_sum) into the caller's three statistics
+  int stats_write(int n) {
+    k_batch_stats<<<1, 256, 0, st>>>(ws.lpart, n, (double)pb.B * NN, pb.stats_out, ws.status);
     PTY_LAUNCH_CHECK("k_batch_stats", -1);
     return PTY_OK;
   }

@@ -73,6 +73,7 @@ size_t layout_workspace(const pty_geom& g, int B, int mode, char* base, Workspac
   const bool want_probe = grad && (g.grad_mask & PTY_GRAD_PROBE);
   const int K = effective_stride(g);
   const int nseg = (g.Nz + K - 1) / K;
+  const size_t loss_ctas = (size_t)(B > 0 ? B : 1) * (g.N / 32);
   size_t off = 0;
   Workspace w;
   memset(&w, 0, sizeof(w));
@@ -89,7 +90,7 @@ size_t layout_workspace(const pty_geom& g, int B, int mode, char* base, Workspac
   w.Imode = (float*)take(sizeof(float) * waves * NN);
   if (mode == MODE_STATS) {
     w.u = (float*)take(sizeof(float) * (size_t)B * NN);
-    w.lpart = (double*)take(sizeof(double) * 2 * (size_t)(B > 0 ? B : 1));
+    w.lpart = (double*)take(sizeof(double) * 2 * loss_ctas);
   }
   if (grad) {
     if (K == 1) {
@@ -103,13 +104,13 @@ size_t layout_workspace(const pty_geom& g, int B, int mode, char* base, Workspac
     }
     w.Psi = (float2*)take(sizeof(float2) * waves * NN);
     w.u = (float*)take(sizeof(float) * (size_t)B * NN);
-    w.lpart = (double*)take(sizeof(double) * 2 * (size_t)(B > 0 ? B : 1));
+    w.lpart = (double*)take(sizeof(double) * 2 * loss_ctas);
     if (want_obj) w.gT = (float2*)take(sizeof(float2) * nobj);
     if (want_probe) w.gPhat = (float2*)take(sizeof(float2) * g.M * NN);
     w.spart = (double*)take(sizeof(double) * 5 * (waves > 0 ? waves : 1));
     if (g.w_pacbed > 0.f) {
       w.pac = (float*)take(sizeof(float) * 3 * NN);
-      w.pacpart = (double*)take(sizeof(double) * (size_t)(B > 0 ? B : 1));
+      w.pacpart = (double*)take(sizeof(double) * loss_ctas);
     }
     if (g.w_sparse > 0.f) {
       w.sppart = (double*)take(sizeof(double) * 152 * 8);
@@ -239,9 +240,9 @@ static int prepare(const pty_geom* g, int B, int mode, const int32_t* idx, const
   return PTY_OK;
 }
 
-// Clears the status word, then runs the pipeline.  First CUDA call of every entry point.
+// Clears the status word and the counter after it, then runs the pipeline.  First CUDA call of every entry point.
 static int dispatch(const Problem& pb) {
-  if (cudaMemsetAsync(pb.ws.status, 0, sizeof(int), pb.stream) != cudaSuccess) {
+  if (cudaMemsetAsync(pb.ws.status, 0, 2 * sizeof(int), pb.stream) != cudaSuccess) {
     set_error("cudaMemsetAsync failed: %s", cudaGetErrorString(cudaGetLastError()));
     return PTY_ECUDA;
   }
@@ -554,10 +555,15 @@ int pty_supported_sizes(void) { return (1 << 6) | (1 << 7) | (1 << 8); }
 
 namespace {
 constexpr size_t kNoallocBytes = (size_t)PTY_NOALLOC_SCRATCH_BYTES;
-// Room on top for the batch entries' table constants, which do not count against the documented limit: a
-// pattern's intensities alone take 4 * 64^2 bytes, so a batch under it has at most 2048 entries.
-size_t wave_const_bytes(int B) { return align_up(sizeof(float) * kWaveConstFloats * (size_t)(B > 0 ? B : 1)); }
-constexpr size_t kNoallocExtra = sizeof(float) * kWaveConstFloats * 2048 + 256;
+// Room on top for the batch entries' table constants and the loss kernel's sums beyond one per pattern, which do
+// not count against the documented limit: a pattern's intensities alone take 4 N^2 bytes, so a batch
+// under it has at most 2048 entries at N = 64, 512 at 128, 128 at 256.
+size_t extra_bytes(const pty_geom& g, int B) {
+  const size_t n = B > 0 ? B : 1, parts = g.N / 32;
+  return align_up(sizeof(float) * kWaveConstFloats * n) + (align_up(16 * n * parts) - align_up(16 * n)) +
+         (g.w_pacbed > 0.f ? align_up(8 * n * parts) - align_up(8 * n) : 0);
+}
+constexpr size_t kNoallocExtra = (sizeof(float) * kWaveConstFloats + 64) * 2048;
 // Loaded with the library's device code on every GPU that uses it and held until the process exits.
 __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocBytes + kNoallocExtra];
 // Device address of g_noalloc_scratch per device ordinal (host code may not use the symbol itself).
@@ -577,9 +583,9 @@ int pty_loss_grad_noalloc(const pty_geom* geom, int B, const int32_t* idx, const
   int rc = validate_geom(geom);
   if (rc) return rc;
   REQUIRE(B >= 0, "batch size %d < 0", B);
-  const size_t need = layout_workspace(*geom, B, MODE_GRAD, nullptr, nullptr) - wave_const_bytes(B);
+  const size_t need = layout_workspace(*geom, B, MODE_GRAD, nullptr, nullptr) - extra_bytes(*geom, B);
   if (need > kNoallocBytes) {
-    const size_t empty = layout_workspace(*geom, 0, MODE_GRAD, nullptr, nullptr) - wave_const_bytes(0);
+    const size_t empty = layout_workspace(*geom, 0, MODE_GRAD, nullptr, nullptr) - extra_bytes(*geom, 0);
     if (empty > kNoallocBytes)
       set_error("pty_loss_grad_noalloc: the object alone needs %zu bytes of scratch (transmission and its "
                 "gradient) but the fixed area holds %zu; no batch fits; use pty_loss_grad with a caller-owned "

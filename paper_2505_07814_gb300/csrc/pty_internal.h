@@ -13,7 +13,7 @@ namespace pty {
 struct Pair;       // pipeline.cuh
 constexpr int kWaveConstFloats = 16;
 struct Workspace {
-  int* status;     // [1]   device status bits
+  int* status;     // [2]   device status bits; the loss kernel's count of finished CTAs
   Pair* wc;        // [B][8] pairs of floats: constants of each batch entry's propagator tables
   float2* T;       // [Ko][Nz][H][W]  transmission amp * exp(i phase)
   float2* Phat;    // [M][N*N]        probe spectra F[P_m] (k-space layout)
@@ -26,7 +26,7 @@ struct Workspace {
   float2* Psi;     // [B][M][N*N]     far-field waves (k-space)
   float* Imode;    // [B][M][N*N]     per-mode far-field intensity (k-space)
   float* u;        // [B][N*N]        dL/dI before the batch normaliser (k-space)
-  double* lpart;   // [B][2]          per-pattern loss sums
+  double* lpart;   // [B][N / 32][2]  loss sums of the loss kernel's CTAs
   double* scal;    // [4]             {dL/dI normaliser, loss, -, -}
   float2* gT;      // [Ko][Nz][H][W]  dL/dT accumulator
   float2* gPhat;   // [M][N*N]        probe-spectrum gradient accumulator (k-space)
@@ -36,8 +36,8 @@ struct Workspace {
   float2* tmp;     // [B][M][N*N]     half-transformed waves (transposed per wave)
   float* gscal;    // [4]             fp16 batch scaling: {max |x| bits, scale, -, -}
   // extra loss terms (when their weights are non-zero)
-  float* pac;      // [3][N*N]        sum over the batch of I_model, of I_meas (k-space), PACBED dL/dI
-  double* pacpart; // [B]             per-pattern sums of I_meas^p_pacbed
+  float* pac;      // [3][N*N]        sum over the batch of I_model, of I_meas (detector order), PACBED dL/dI
+  double* pacpart; // [B][N / 32]     sums of I_meas^p_pacbed
   double* sppart;  // [152*8]         partial sums of c |phase|^p_sparse (sparsity term)
   int* cover;      // [H][W+1]        patch coverage count c of the batch (sparsity term)
   void* pieces0;   // [B][M][N][pieces][2N] 16-bit split operands of the tensor-core GEMMs
