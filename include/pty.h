@@ -310,7 +310,9 @@ int pty_loss_grad_noalloc(const pty_geom* geom, int B, const int32_t* idx, const
  * pty_profile_read fills ms[k] with the summed device time of pipeline stage k over the recorded
  *   calls, for k < min(n, PTY_PROF_STAGES), synchronising on the recorded events; returns the number
  *   of calls recorded, or -1 on a CUDA error.  Stages: 0 prepare_object, 1 probe_spectrum, 2 forward,
- *   3 loss, 4 loss_finalize, 5 adjoint, 6 object_grad, 7 probe_grad, 8 scalar_grad. */
+ *   3 loss, 4 loss_finalize, 5 adjoint, 6 object_grad, 7 probe_grad, 8 scalar_grad.  Work that shares
+ *   a launch is counted in the first of its stages (0 holds 1 and 6 holds 7 and 8 for objects up to
+ *   8 Mi voxels at N <= 128; 3 always holds 4). */
 #define PTY_PROF_STAGES 9
 long long pty_launch_count(void);
 int pty_profile_enable(int on);

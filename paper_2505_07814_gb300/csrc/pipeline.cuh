@@ -3,20 +3,20 @@
 // loop; the wave never leaves shared memory except as checkpoints for the adjoint.
 //
 // Kernel sequence of one pty_loss_grad call (one stream, no host synchronisation):
-//   k_prepare          T = amp exp(i phase) for the whole object; the constants of every batch
-//                      entry's tables
-//   k_probe_spectrum   P^_m = F[P_m]                                              (M CTAs)
+//   k_begin            T = amp exp(i phase) for the whole object, the constants of every batch entry's tables,
+//                      zeroed accumulators; P^_m = F[P_m]
 //   k_forward          shift, Nz transmissions, Nz-1 propagations, far field      (B*M CTAs)
 //   k_loss             mode sum, Eq. 5/6 per pixel, dL/dI; the last CTA forms the batch loss and the dL/dI
 //                      normaliser (FP64)                                      (B * N / 32 CTAs)
 //   k_adjoint          reverse of k_forward, scatter-adds dL/dT, probe-spectrum
 //                      gradient, FP64-reduced position / tilt / dz partials       (B*M CTAs)
-//   k_object_grad      dL/damp, dL/dphase from dL/dT (chain rule of amp exp(i phase))
-//   k_probe_grad       dL/dP_m = F^-1[accumulated spectrum gradient]              (M CTAs)
-//   k_scalar_grad      positions, tilts, dz from the per-wave partials
+//   k_finish           dL/damp, dL/dphase from dL/dT (chain rule of amp exp(i phase)); dL/dP_m =
+//                      F^-1[accumulated spectrum gradient]; positions, tilts, dz from the per-wave partials
+// (k_begin and k_finish as three kernels each for clusters and large objects).
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
+#include <string.h>
 
 #include "fft_cluster.cuh"
 #include "fft_smem.cuh"
@@ -295,14 +295,20 @@ enum { WC_K2, WC_K0, WC_K1, WC_E2, WC_E0, WC_E1, WC_C0, WC_C1, kWaveConsts };
 static_assert(kWaveConsts * 2 == kWaveConstFloats, "workspace layout");
 
 // ---------------------------------------------------------------------------------------------
-// Start of a forward: object transmission (blocks 0 .. blocks - 1) and, by the blocks after them, the
-// constants of every batch entry, four threads an entry (its tangents and cosines are chains of some
-// hundred FP64 instructions, so each has a thread of its own).
+// Start of a forward: object transmission and zeroed accumulators (blocks 0 .. blocks - 1) and, by the blocks
+// after them, the constants of every batch entry, four threads an entry (its tangents and cosines are
+// chains of some hundred FP64 instructions, so each has a thread of its own).
 // ---------------------------------------------------------------------------------------------
 struct PrepArgs {
   const float *amp, *phase;
   float2* T;
+  float2* gT;  // zeroed with T when given
   size_t n;
+  int vec;     // n a multiple of 4 and the arrays 16-byte aligned
+  struct {
+    float* p;
+    size_t n;
+  } zero[4];   // further arrays to zero
   int blocks;  // of the object part
   int B, Ntot, global_tilt;
   double lam, kq;
@@ -311,9 +317,12 @@ struct PrepArgs {
   Pair* wc;  // [B][kWaveConsts]
   int* status;
 };
-static __global__ void __launch_bounds__(256) k_prepare(PrepArgs a) {
-  if ((int)blockIdx.x >= a.blocks) {
-    const int t = (blockIdx.x - a.blocks) * 256 + threadIdx.x, part = t / 32 & 3, b = (t / 128) * 32 + (t & 31);
+// blocks of T threads that hold the constants' part (threads in groups of 128 for 32 entries)
+__host__ __device__ constexpr int prep_const_blocks(int B, int T) { return (B + T / 4 - 1) / (T / 4); }
+template <int T>
+__device__ __forceinline__ void prepare_part(const PrepArgs& a, int block) {
+  if (block >= a.blocks) {
+    const int t = (block - a.blocks) * T + threadIdx.x, part = t / 32 & 3, b = (t / 128) * 32 + (t & 31);
     if (b >= a.B) return;
     int j = a.idx[b];
     if (j < 0 || j >= a.Ntot) {
@@ -335,38 +344,83 @@ static __global__ void __launch_bounds__(256) k_prepare(PrepArgs a) {
     }
     return;
   }
-  for (size_t i = blockIdx.x * (size_t)256 + threadIdx.x; i < a.n; i += (size_t)a.blocks * 256) {
-    float s, c;
-    sincosf(a.phase[i], &s, &c);
-    const float m = a.amp[i];
-    a.T[i] = make_float2(m * c, m * s);
+  const size_t first = block * (size_t)T + threadIdx.x, step = (size_t)a.blocks * T;
+  if (a.vec) {
+    for (size_t i = first; i < a.n / 4; i += step) {
+      const float4 ph = reinterpret_cast<const float4*>(a.phase)[i], m = reinterpret_cast<const float4*>(a.amp)[i];
+      float4 s, c;
+      sincosf(ph.x, &s.x, &c.x);
+      sincosf(ph.y, &s.y, &c.y);
+      sincosf(ph.z, &s.z, &c.z);
+      sincosf(ph.w, &s.w, &c.w);
+      float4* t = reinterpret_cast<float4*>(a.T) + 2 * i;
+      t[0] = make_float4(m.x * c.x, m.x * s.x, m.y * c.y, m.y * s.y);
+      t[1] = make_float4(m.z * c.z, m.z * s.z, m.w * c.w, m.w * s.w);
+      if (a.gT) {
+        float4* g = reinterpret_cast<float4*>(a.gT) + 2 * i;
+        g[0] = g[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    }
+  } else {
+    for (size_t i = first; i < a.n; i += step) {
+      float s, c;
+      sincosf(a.phase[i], &s, &c);
+      const float m = a.amp[i];
+      a.T[i] = make_float2(m * c, m * s);
+      if (a.gT) a.gT[i] = make_float2(0.f, 0.f);
+    }
   }
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    for (size_t i = first; i < a.zero[k].n; i += step) a.zero[k].p[i] = 0.f;
 }
+static __global__ void __launch_bounds__(256) k_prepare(PrepArgs a) { prepare_part<256>(a, blockIdx.x); }
 
 // ---------------------------------------------------------------------------------------------
-// Probe spectra P^_m = F[P_m] (k-space layout); zero the probe-gradient accumulator.
+// Probe spectra P^_m = F[P_m] (k-space layout), one CTA (cluster) per mode.
 // ---------------------------------------------------------------------------------------------
+// A thread's elements tid + T i are loaded 16 at a time: one after the other, their latencies were most of
+// the kernel (N = 64, one mode: 5.6 us).
+template <int N, int T, class Load, class Store>
+__device__ __forceinline__ void each_element(Load&& load, Store&& store) {
+  constexpr int n = wave_rows<N>() * N / T, U = n < 16 ? n : 16;
+  static_assert(n % U == 0, "elements per thread");
+#pragma unroll 1
+  for (int i0 = 0; i0 < n; i0 += U) {
+    float2 v[U];
+#pragma unroll
+    for (int i = 0; i < U; ++i) v[i] = load(threadIdx.x + T * (i0 + i));
+#pragma unroll
+    for (int i = 0; i < U; ++i) store(threadIdx.x + T * (i0 + i), v[i]);
+  }
+}
 template <int N, int T>
-__global__ void __launch_bounds__(T) k_probe_spectrum(const float2* __restrict__ probe, float2* __restrict__ Phat,
-                                                      float2* __restrict__ gPhat) {
+__device__ __forceinline__ void spectrum_part(const float2* __restrict__ probe, float2* __restrict__ Phat, int block) {
   using F = Fft2<N, T>;
   constexpr int RS = F::RS, R = F::ROWS;
   extern __shared__ __align__(16) float2 sm[];
   float2* s = sm;
   float2* tw = s + R * RS;
-  const int m = blockIdx.x / F::C, q = F::rank(), tid = threadIdx.x;
+  const int m = block / F::C, q = F::rank();
   build_twiddles<N>(tw);
   const float2* P = probe + (size_t)m * N * N + (size_t)q * R * N;  // this CTA's rows of mode m
-  for (int e = tid; e < R * N; e += T) s[(e / N) * RS + e % N] = P[e];
+  each_element<N, T>([&](int e) { return P[e]; }, [&](int e, float2 v) { s[(e / N) * RS + e % N] = v; });
   __syncthreads();
   F::forward(s, tw);
   float2* out = Phat + (size_t)m * N * N;
-  float2* g = gPhat ? gPhat + (size_t)m * N * N : nullptr;
-  for (int e = tid; e < R * N; e += T) {  // local k-space row e % R, column e / R
-    const int k = kidx<N>(q * R + e % R, e / R);
-    out[k] = s[(e % R) * RS + e / R];
-    if (g) g[k] = make_float2(0.f, 0.f);
-  }
+  each_element<N, T>([&](int e) { return s[(e % R) * RS + e / R]; },  // local k-space row e % R, column e / R
+                     [&](int e, float2 v) { out[kidx<N>(q * R + e % R, e / R)] = v; });
+}
+template <int N, int T>
+__global__ void __launch_bounds__(T) k_probe_spectrum(const float2* __restrict__ probe, float2* __restrict__ Phat) {
+  spectrum_part<N, T>(probe, Phat, blockIdx.x);
+}
+// The probe spectra (CTAs 0 .. M - 1) and the rest of a forward's start in one launch.
+template <int N, int T>
+__global__ void __launch_bounds__(T) k_begin(PrepArgs a, const float2* __restrict__ probe, float2* __restrict__ Phat,
+                                             int M) {
+  if ((int)blockIdx.x < M) spectrum_part<N, T>(probe, Phat, blockIdx.x);
+  else prepare_part<T>(a, (int)blockIdx.x - M);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1823,91 +1877,151 @@ static __global__ void k_sparse_grad(const float* __restrict__ phase, const int*
 // Finalisers
 // ---------------------------------------------------------------------------------------------
 // dL/damp = Re(conj(e^{i phase}) dL/dT), dL/dphase = Re(conj(i T) dL/dT) = Im(conj(T) dL/dT)
-static __global__ void k_object_grad(const float* __restrict__ amp, const float* __restrict__ phase,
-                              const float2* __restrict__ gT, float* __restrict__ g_amp, float* __restrict__ g_phase,
-                              int accumulate, size_t n) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    float s, c;
-    sincosf(phase[i], &s, &c);
-    const float2 g = gT[i];
-    const float a = amp[i];
-    const float ga = fmaf(c, g.x, s * g.y);
-    const float gp = a * fmaf(c, g.y, -s * g.x);
-    if (g_amp) g_amp[i] = accumulate ? g_amp[i] + ga : ga;
-    if (g_phase) g_phase[i] = accumulate ? g_phase[i] + gp : gp;
+struct ObjGradArgs {
+  const float *amp, *phase;
+  const float2* gT;
+  float *g_amp, *g_phase;  // or nullptr
+  int accumulate, vec;     // vec: as PrepArgs
+  size_t n;
+  int blocks;
+};
+__device__ __forceinline__ float2 object_grad(float a, float ph, float2 g) {
+  float s, c;
+  sincosf(ph, &s, &c);
+  return make_float2(fmaf(c, g.x, s * g.y), a * fmaf(c, g.y, -s * g.x));
+}
+template <int T>
+__device__ __forceinline__ void object_grad_part(const ObjGradArgs& o, int block) {
+  const size_t first = block * (size_t)T + threadIdx.x, step = (size_t)o.blocks * T;
+  if (o.vec) {
+    for (size_t i = first; i < o.n / 4; i += step) {
+      const float4 a = reinterpret_cast<const float4*>(o.amp)[i], p = reinterpret_cast<const float4*>(o.phase)[i];
+      const float4 g0 = reinterpret_cast<const float4*>(o.gT)[2 * i], g1 = reinterpret_cast<const float4*>(o.gT)[2 * i + 1];
+      const float2 v0 = object_grad(a.x, p.x, make_float2(g0.x, g0.y)), v1 = object_grad(a.y, p.y, make_float2(g0.z, g0.w));
+      const float2 v2 = object_grad(a.z, p.z, make_float2(g1.x, g1.y)), v3 = object_grad(a.w, p.w, make_float2(g1.z, g1.w));
+      float4 ga = make_float4(v0.x, v1.x, v2.x, v3.x), gp = make_float4(v0.y, v1.y, v2.y, v3.y);
+      float4* A = reinterpret_cast<float4*>(o.g_amp) + i;
+      float4* P = reinterpret_cast<float4*>(o.g_phase) + i;
+      if (o.g_amp) {
+        if (o.accumulate) {
+          const float4 x = *A;
+          ga = make_float4(x.x + ga.x, x.y + ga.y, x.z + ga.z, x.w + ga.w);
+        }
+        *A = ga;
+      }
+      if (o.g_phase) {
+        if (o.accumulate) {
+          const float4 x = *P;
+          gp = make_float4(x.x + gp.x, x.y + gp.y, x.z + gp.z, x.w + gp.w);
+        }
+        *P = gp;
+      }
+    }
+    return;
+  }
+  for (size_t i = first; i < o.n; i += step) {
+    const float2 v = object_grad(o.amp[i], o.phase[i], o.gT[i]);
+    if (o.g_amp) o.g_amp[i] = o.accumulate ? o.g_amp[i] + v.x : v.x;
+    if (o.g_phase) o.g_phase[i] = o.accumulate ? o.g_phase[i] + v.y : v.y;
   }
 }
+static __global__ void __launch_bounds__(256) k_object_grad(ObjGradArgs o) { object_grad_part<256>(o, blockIdx.x); }
 
 // The accumulator holds A = sum_j conj(R_j) F[dL/dP_j] (R_j the shift ramp of position j).  The
 // probe-spectrum gradient is A / N^2 and dL/dP_m = F^H[A / N^2] = (plain inverse sum of A) / N^2.
 template <int N, int T>
-__global__ void __launch_bounds__(T) k_probe_grad(const float2* __restrict__ gPhat, float2* __restrict__ g_probe,
-                                                  int accumulate) {
+__device__ __forceinline__ void probe_grad_part(const float2* __restrict__ gPhat, float2* __restrict__ g_probe,
+                                                int accumulate, int block) {
   using F = Fft2<N, T>;
   constexpr int RS = F::RS;
   extern __shared__ __align__(16) float2 sm[];
   float2* s = sm;
   float2* tw = s + F::ROWS * RS;
-  const int m = blockIdx.x / F::C, q = F::rank(), tid = threadIdx.x;
+  const int m = block / F::C, q = F::rank();
   constexpr int R = F::ROWS;
   build_twiddles<N>(tw);
   const float2* G = gPhat + (size_t)m * N * N;
-  for (int e = tid; e < R * N; e += T) s[(e % R) * RS + e / R] = G[kidx<N>(q * R + e % R, e / R)];
+  each_element<N, T>([&](int e) { return G[kidx<N>(q * R + e % R, e / R)]; },
+                     [&](int e, float2 v) { s[(e % R) * RS + e / R] = v; });
   __syncthreads();
   F::inverse(s, tw);
   const float sc = 1.0f / (float)(N * N);
   float2* out = g_probe + (size_t)m * N * N + (size_t)q * R * N;  // this CTA's rows
-  for (int e = tid; e < R * N; e += T) {
-    const float2 v = cscale(s[(e / N) * RS + e % N], sc);
-    out[e] = accumulate ? cadd(out[e], v) : v;
-  }
+  if (accumulate)
+    each_element<N, T>([&](int e) { return cadd(out[e], cscale(s[(e / N) * RS + e % N], sc)); },
+                       [&](int e, float2 v) { out[e] = v; });
+  else
+    each_element<N, T>([&](int e) { return cscale(s[(e / N) * RS + e % N], sc); }, [&](int e, float2 v) { out[e] = v; });
+}
+template <int N, int T>
+__global__ void __launch_bounds__(T) k_probe_grad(const float2* __restrict__ gPhat, float2* __restrict__ g_probe,
+                                                  int accumulate) {
+  probe_grad_part<N, T>(gPhat, g_probe, accumulate, blockIdx.x);
 }
 
-// Positions, tilts (summed over modes; over positions too for a global tilt) and dz.
-static __global__ void k_scalar_grad(const double* __restrict__ spart, const int32_t* __restrict__ idx, int B, int M,
-                              int Ntot, int global_tilt, int grad_mask, float* g_pos, float* g_tilt, float* g_dz,
-                              int accumulate) {
-  __shared__ double red[64];
-  double dzs = 0.0, t0s = 0.0;
-  double t1s = 0.0;
-  for (int b = threadIdx.x; b < B; b += blockDim.x) {
+// Positions, tilts (summed over modes; over positions too for a global tilt) and dz: one CTA.
+struct ScalarArgs {
+  const double* spart;
+  const int32_t* idx;
+  int B, M, Ntot, global_tilt, grad_mask;  // M: waves per position
+  float *g_pos, *g_tilt, *g_dz;
+  int accumulate;
+};
+template <int T>
+__device__ __forceinline__ void scalar_grad_part(const ScalarArgs& a) {
+  __shared__ double red[2 * (T / 32)];
+  double dzs = 0.0, t0s = 0.0, t1s = 0.0;
+  for (int b = threadIdx.x; b < a.B; b += T) {
     double p0 = 0.0, p1 = 0.0, a0 = 0.0, a1 = 0.0;
-    for (int m = 0; m < M; ++m) {
-      const double* sp = spart + ((size_t)b * M + m) * 5;
+#pragma unroll 4
+    for (int m = 0; m < a.M; ++m) {
+      const double* sp = a.spart + ((size_t)b * a.M + m) * 5;
       p0 += sp[0];
       p1 += sp[1];
       a0 += sp[2];
       a1 += sp[3];
       dzs += sp[4];
     }
-    const int j = idx[b];
-    if (j < 0 || j >= Ntot) continue;  // flagged by the forward kernel
-    if ((grad_mask & PTY_GRAD_POS) && g_pos) {
-      atomicAdd(g_pos + 2 * j, (float)p0);
-      atomicAdd(g_pos + 2 * j + 1, (float)p1);
+    const int j = a.idx[b];
+    if (j < 0 || j >= a.Ntot) continue;  // flagged by the forward kernel
+    if ((a.grad_mask & PTY_GRAD_POS) && a.g_pos) {
+      atomicAdd(a.g_pos + 2 * j, (float)p0);
+      atomicAdd(a.g_pos + 2 * j + 1, (float)p1);
     }
-    if ((grad_mask & PTY_GRAD_TILT) && g_tilt) {
-      if (global_tilt) {
+    if ((a.grad_mask & PTY_GRAD_TILT) && a.g_tilt) {
+      if (a.global_tilt) {
         t0s += a0;
         t1s += a1;
       } else {
-        atomicAdd(g_tilt + 2 * j, (float)a0);
-        atomicAdd(g_tilt + 2 * j + 1, (float)a1);
+        atomicAdd(a.g_tilt + 2 * j, (float)a0);
+        atomicAdd(a.g_tilt + 2 * j + 1, (float)a1);
       }
     }
   }
   double x = dzs, y = t0s;
-  block_sum2<256>(x, y, red);
+  block_sum2<T>(x, y, red);
   __syncthreads();
   double z = t1s, dummy = 0.0;
-  block_sum2<256>(z, dummy, red);
+  block_sum2<T>(z, dummy, red);
   if (threadIdx.x == 0) {
-    if ((grad_mask & PTY_GRAD_DZ) && g_dz) g_dz[0] = accumulate ? g_dz[0] + (float)x : (float)x;
-    if ((grad_mask & PTY_GRAD_TILT) && g_tilt && global_tilt) {
-      g_tilt[0] = accumulate ? g_tilt[0] + (float)y : (float)y;
-      g_tilt[1] = accumulate ? g_tilt[1] + (float)z : (float)z;
+    if ((a.grad_mask & PTY_GRAD_DZ) && a.g_dz) a.g_dz[0] = a.accumulate ? a.g_dz[0] + (float)x : (float)x;
+    if ((a.grad_mask & PTY_GRAD_TILT) && a.g_tilt && a.global_tilt) {
+      a.g_tilt[0] = a.accumulate ? a.g_tilt[0] + (float)y : (float)y;
+      a.g_tilt[1] = a.accumulate ? a.g_tilt[1] + (float)z : (float)z;
     }
   }
+}
+static __global__ void __launch_bounds__(256) k_scalar_grad(ScalarArgs a) { scalar_grad_part<256>(a); }
+
+// All three in one launch: CTAs 0 .. M - 1 the probe modes (M = 0: none), CTA M the scalars when `scalars`, the others
+// the object.
+template <int N, int T>
+__global__ void __launch_bounds__(T) k_finish(ObjGradArgs o, ScalarArgs a, int scalars, const float2* __restrict__ gPhat,
+                                              float2* __restrict__ g_probe, int M) {
+  const int block = blockIdx.x;
+  if (block < M) probe_grad_part<N, T>(gPhat, g_probe, a.accumulate, block);
+  else if (scalars && block == M) scalar_grad_part<T>(a);
+  else object_grad_part<T>(o, block - M - scalars);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1987,24 +2101,32 @@ struct Pass {
   auto recompute_kernel() const { return pb.Ko > 1 ? k_recompute<N, TF, true> : k_recompute<N, TF, false>; }
   auto adj_kernel() const { return pb.Ko > 1 ? k_adjoint<N, TA, true> : k_adjoint<N, TA, false>; }
 
+  // Launch attributes of this size's kernels, set once per device (they belong to the loaded functions; two
+  // threads that meet here set the same values).
   int set_attributes() {
-    bool ok = cudaFuncSetAttribute(fwd_kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)fwd_kernel_smem_bytes<N>()) == cudaSuccess &&
-              cudaFuncSetAttribute(recompute_kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)fwd_smem_bytes<N>()) == cudaSuccess &&
-              cudaFuncSetAttribute(adj_kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)adj_smem_bytes<N, TA>()) == cudaSuccess &&
-              cudaFuncSetAttribute(k_probe_spectrum<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)probe_smem()) == cudaSuccess &&
-              cudaFuncSetAttribute(k_probe_grad<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)probe_smem()) == cudaSuccess;
+    static bool ready[2][256] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 256) {
+      set_error("no current CUDA device");
+      return PTY_ECUDA;
+    }
+    bool* done = &ready[pb.Ko > 1][dev];
+    if (__atomic_load_n(done, __ATOMIC_ACQUIRE)) return PTY_OK;
+    auto smem = [](auto kern, size_t bytes) {
+      return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+    };
+    bool ok = smem(fwd_kernel(), fwd_kernel_smem_bytes<N>()) && smem(recompute_kernel(), fwd_smem_bytes<N>()) &&
+              smem(adj_kernel(), adj_smem_bytes<N, TA>());
+    if constexpr (C == 1) {
+      ok = ok && smem(k_begin<N, T>, probe_smem()) && smem(k_finish<N, T>, probe_smem());
+    }
+    ok = ok && smem(k_probe_spectrum<N, T>, probe_smem()) && smem(k_probe_grad<N, T>, probe_smem());
 #if PTY_CARVEOUT
     // One N = 128 wave kernel CTA per SM: ask for the smallest shared-memory carve-out that holds it,
     // so the rest of the SM's on-chip memory serves as L1 for the loads in flight.
     if constexpr (N == 128) {
-      int dev = 0, smem_sm = 0;
-      ok = ok && cudaGetDevice(&dev) == cudaSuccess &&
-           cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) == cudaSuccess &&
+      int smem_sm = 0;
+      ok = ok && cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) == cudaSuccess &&
            smem_sm > 0;
       auto pct = [&](size_t bytes) { return (int)((100 * (bytes + 1024) + smem_sm - 1) / (size_t)smem_sm); };
       ok = ok &&
@@ -2018,13 +2140,24 @@ struct Pass {
       set_error("cudaFuncSetAttribute failed: %s", cudaGetErrorString(cudaGetLastError()));
       return PTY_ECUDA;
     }
+    __atomic_store_n(done, true, __ATOMIC_RELEASE);
     return PTY_OK;
   }
   static size_t probe_smem() { return sizeof(float2) * ((size_t)wave_rows<N>() * (N + 1) + N); }
+  size_t nobj() const { return (size_t)pb.Ko * pb.Nz * pb.H * pb.W; }
   unsigned object_blocks() const {
-    const size_t nobj = (size_t)pb.Ko * pb.Nz * pb.H * pb.W;
-    return (unsigned)((nobj + 255) / 256 < 152 * 16 ? (nobj + 255) / 256 : 152 * 16);
+    return (unsigned)((nobj() + 255) / 256 < 152 * 16 ? (nobj() + 255) / 256 : 152 * 16);
   }
+  // Whether the object's passes share a launch with the probe's transforms.  The launch then has the
+  // transforms' shared memory, so an SM holds few of its CTAs; that costs nothing while the object's
+  // arrays fit L2 (8 Mi voxels: 64 MB of T), and saves a launch and the wait between two small kernels
+  // (64 x 64, one mode, 128 x 128 object: 3.3 + 5.6 us as two kernels, 3.8 as one).
+  bool together() const { return C == 1 && nobj() <= ((size_t)8 << 20); }
+  unsigned shared_blocks() const {  // CTAs of T threads for the object in such a launch, four elements a thread
+    const size_t b = (nobj() + 4 * T - 1) / (4 * T), per = N == 64 ? 4 : 1;
+    return (unsigned)(b < 152 * per ? b : 152 * per);
+  }
+  static bool quad(const void* p) { return aligned(p, 16); }
 
   FwdArgs fwd_args() const {
     FwdArgs fa;
@@ -2055,11 +2188,12 @@ struct Pass {
   int forward_begin() {
     prof_begin(st);
     PrepArgs pa;
+    memset(&pa, 0, sizeof(pa));
     pa.amp = pb.amp;
     pa.phase = pb.phase;
     pa.T = ws.T;
-    pa.n = (size_t)pb.Ko * pb.Nz * pb.H * pb.W;
-    pa.blocks = (int)object_blocks();
+    pa.n = nobj();
+    pa.vec = pa.n % 4 == 0 && quad(pb.amp) && quad(pb.phase);
     pa.B = pb.B;
     pa.Ntot = pb.Ntot;
     pa.global_tilt = pb.global_tilt;
@@ -2070,10 +2204,31 @@ struct Pass {
     pa.dz = pb.dz;
     pa.wc = ws.wc;
     pa.status = ws.status;
-    k_prepare<<<pa.blocks + (pb.B + 63) / 64, 256, 0, st>>>(pa);
+    if (zeroes_early()) {
+      const int gm = pb.grad_mask;
+      int k = 0;
+      auto clear = [&](void* p, size_t bytes) {
+        pa.zero[k].p = (float*)p;
+        pa.zero[k++].n = bytes / sizeof(float);
+      };
+      if (want_obj) pa.gT = ws.gT;
+      if (want_probe) clear(ws.gPhat, sizeof(float2) * pb.M * NN);
+      clear(ws.spart, sizeof(double) * 5 * pb.B * pb.M * pb.Ko);
+      if (!pb.accumulate && (gm & PTY_GRAD_POS)) clear(pb.g_pos, sizeof(float) * 2 * pb.Ntot);
+      if (!pb.accumulate && (gm & PTY_GRAD_TILT) && !pb.global_tilt) clear(pb.g_tilt, sizeof(float) * 2 * pb.Ntot);
+    }
+    if constexpr (C == 1) {
+      if (together()) {
+        pa.blocks = (int)shared_blocks();
+        k_begin<N, T><<<pb.M + pa.blocks + prep_const_blocks(pb.B, T), T, probe_smem(), st>>>(pa, pb.probe, ws.Phat, pb.M);
+        PTY_LAUNCH_CHECK("k_begin", 0);
+        return PTY_OK;
+      }
+    }
+    pa.blocks = (int)object_blocks();
+    k_prepare<<<pa.blocks + prep_const_blocks(pb.B, 256), 256, 0, st>>>(pa);
     PTY_LAUNCH_CHECK("k_prepare", 0);
-    PTY_LAUNCH_RC(launch_waves<C>(k_probe_spectrum<N, T>, pb.M, T, probe_smem(), st, pb.probe, ws.Phat,
-                                   (float2*)nullptr),
+    PTY_LAUNCH_RC(launch_waves<C>(k_probe_spectrum<N, T>, pb.M, T, probe_smem(), st, pb.probe, ws.Phat),
                   "k_probe_spectrum", 1);
     return PTY_OK;
   }
@@ -2197,14 +2352,21 @@ struct Pass {
     return aa;
   }
 
+  // A pass that runs its own adjoint has the forward's first kernel zero what the adjoint adds into.
+  bool zeroes_early() const { return pb.mode == MODE_GRAD; }
   // Zero the accumulators of the adjoint.
   int adjoint_begin() {
-    const size_t nobj = (size_t)pb.Ko * pb.Nz * pb.H * pb.W;
-    if (want_obj && cudaMemsetAsync(ws.gT, 0, sizeof(float2) * nobj, st) != cudaSuccess) return memset_failed();
-    if (want_probe && cudaMemsetAsync(ws.gPhat, 0, sizeof(float2) * pb.M * NN, st) != cudaSuccess) return memset_failed();
-    if (pb.B > 0 && cudaMemsetAsync(ws.spart, 0, sizeof(double) * 5 * pb.B * pb.M * pb.Ko, st) != cudaSuccess)
-      return memset_failed();
-    return PTY_OK;
+    if (zeroes_early()) return PTY_OK;
+    const int gm = pb.grad_mask;
+    auto clear = [&](void* p, size_t bytes) { return cudaMemsetAsync(p, 0, bytes, st) == cudaSuccess; };
+    bool ok = true;
+    if (want_obj) ok = ok && clear(ws.gT, sizeof(float2) * nobj());
+    if (want_probe) ok = ok && clear(ws.gPhat, sizeof(float2) * pb.M * NN);
+    if (pb.B > 0) ok = ok && clear(ws.spart, sizeof(double) * 5 * pb.B * pb.M * pb.Ko);
+    if (!pb.accumulate && (gm & PTY_GRAD_POS) && pb.g_pos) ok = ok && clear(pb.g_pos, sizeof(float) * 2 * pb.Ntot);
+    if (!pb.accumulate && (gm & PTY_GRAD_TILT) && pb.g_tilt && !pb.global_tilt)
+      ok = ok && clear(pb.g_tilt, sizeof(float) * 2 * pb.Ntot);
+    return ok ? PTY_OK : memset_failed();
   }
 
   // The adjoint kernels over all slices (segment by segment in the recompute mode).
@@ -2256,10 +2418,33 @@ struct Pass {
   // phase-sparsity term of the loss and its gradient.
   int finalize() {
     const int gm = pb.grad_mask;
-    const size_t nobj = (size_t)pb.Ko * pb.Nz * pb.H * pb.W;
-    if (want_obj) {
-      k_object_grad<<<object_blocks(), 256, 0, st>>>(pb.amp, pb.phase, ws.gT, (gm & PTY_GRAD_AMP) ? pb.g_amp : nullptr,
-                                                     (gm & PTY_GRAD_PHASE) ? pb.g_phase : nullptr, pb.accumulate, nobj);
+    const bool scalars = (gm & (PTY_GRAD_POS | PTY_GRAD_TILT | PTY_GRAD_DZ)) && pb.B > 0;
+    ObjGradArgs oa;
+    oa.amp = pb.amp;
+    oa.phase = pb.phase;
+    oa.gT = ws.gT;
+    oa.g_amp = (gm & PTY_GRAD_AMP) ? pb.g_amp : nullptr;
+    oa.g_phase = (gm & PTY_GRAD_PHASE) ? pb.g_phase : nullptr;
+    oa.accumulate = pb.accumulate;
+    oa.n = nobj();
+    oa.vec = oa.n % 4 == 0 && quad(pb.amp) && quad(pb.phase) && quad(oa.g_amp) && quad(oa.g_phase);
+    ScalarArgs sa{ws.spart, pb.idx, pb.B, pb.M * pb.Ko, pb.Ntot, pb.global_tilt, gm, pb.g_pos, pb.g_tilt, pb.g_dz,
+                  pb.accumulate};
+    bool rest = true;  // the probe's and the scalars' gradients have launches of their own
+    if constexpr (C == 1) {
+      if (together()) {
+        oa.blocks = want_obj ? (int)shared_blocks() : 0;
+        const int modes = want_probe ? pb.M : 0, grid = modes + (scalars ? 1 : 0) + oa.blocks;
+        if (grid > 0) {
+          k_finish<N, T><<<grid, T, want_probe ? probe_smem() : 0, st>>>(oa, sa, scalars ? 1 : 0, ws.gPhat, pb.g_probe, modes);
+          PTY_LAUNCH_CHECK("k_finish", 6);
+        }
+        rest = false;
+      }
+    }
+    if (rest && want_obj) {
+      oa.blocks = (int)object_blocks();
+      k_object_grad<<<oa.blocks, 256, 0, st>>>(oa);
       PTY_LAUNCH_CHECK("k_object_grad", 6);
     }
     if (pb.mode == MODE_GRAD && pb.w_sp > 0.f && ws.sppart && pb.B > 0) {
@@ -2271,45 +2456,35 @@ struct Pass {
       k_cover_scan<<<(unsigned)((pb.H + 7) / 8), 256, 0, st>>>(ws.cover, pb.H, pb.W);
       PTY_LAUNCH_CHECK("k_cover_scan", -1);
       const double patch_pixels = (double)pb.B * pb.Ko * pb.Nz * NN;  // the mean's denominator
-      k_sparse_sum<256><<<kSparseBlocks, 256, 0, st>>>(pb.phase, ws.cover, pb.H, pb.W, nobj, pb.p_sp, ws.sppart);
+      k_sparse_sum<256><<<kSparseBlocks, 256, 0, st>>>(pb.phase, ws.cover, pb.H, pb.W, nobj(), pb.p_sp, ws.sppart);
       PTY_LAUNCH_CHECK("k_sparse_sum", -1);
       k_sparse_finalize<<<1, 256, 0, st>>>(ws.sppart, kSparseBlocks, patch_pixels, pb.p_sp, pb.w_sp, pb.loss_out,
                                            ws.scal, ws.status);
       PTY_LAUNCH_CHECK("k_sparse_finalize", -1);
       if ((gm & PTY_GRAD_PHASE) && pb.g_phase) {
         if (!want_obj && !pb.accumulate &&
-            cudaMemsetAsync(pb.g_phase, 0, sizeof(float) * nobj, st) != cudaSuccess)
+            cudaMemsetAsync(pb.g_phase, 0, sizeof(float) * nobj(), st) != cudaSuccess)
           return memset_failed();
-        k_sparse_grad<<<object_blocks(), 256, 0, st>>>(pb.phase, ws.cover, pb.H, pb.W, nobj, pb.p_sp, pb.w_sp,
+        k_sparse_grad<<<object_blocks(), 256, 0, st>>>(pb.phase, ws.cover, pb.H, pb.W, nobj(), pb.p_sp, pb.w_sp,
                                                        ws.scal, pb.g_phase);
         PTY_LAUNCH_CHECK("k_sparse_grad", -1);
       }
     }
-    if (want_probe) {
+    if (rest && want_probe) {
       PTY_LAUNCH_RC(launch_waves<C>(k_probe_grad<N, T>, pb.M, T, probe_smem(), st, (const float2*)ws.gPhat,
                                      pb.g_probe, pb.accumulate),
                     "k_probe_grad", 7);
     }
-    if (gm & (PTY_GRAD_POS | PTY_GRAD_TILT | PTY_GRAD_DZ)) {
-      if (!pb.accumulate) {
-        if ((gm & PTY_GRAD_POS) && pb.g_pos &&
-            cudaMemsetAsync(pb.g_pos, 0, sizeof(float) * 2 * pb.Ntot, st) != cudaSuccess)
-          return memset_failed();
-        if ((gm & PTY_GRAD_TILT) && pb.g_tilt && !pb.global_tilt &&
-            cudaMemsetAsync(pb.g_tilt, 0, sizeof(float) * 2 * pb.Ntot, st) != cudaSuccess)
-          return memset_failed();
-      }
-      if (pb.B > 0) {
-        k_scalar_grad<<<1, 256, 0, st>>>(ws.spart, pb.idx, pb.B, pb.M * pb.Ko, pb.Ntot, pb.global_tilt, gm, pb.g_pos,
-                                         pb.g_tilt, pb.g_dz, pb.accumulate);
-        PTY_LAUNCH_CHECK("k_scalar_grad", 8);
-      } else if (!pb.accumulate) {
-        if ((gm & PTY_GRAD_DZ) && pb.g_dz && cudaMemsetAsync(pb.g_dz, 0, sizeof(float), st) != cudaSuccess)
-          return memset_failed();
-        if ((gm & PTY_GRAD_TILT) && pb.g_tilt && pb.global_tilt &&
-            cudaMemsetAsync(pb.g_tilt, 0, 2 * sizeof(float), st) != cudaSuccess)
-          return memset_failed();
-      }
+    if (rest && scalars) {
+      k_scalar_grad<<<1, 256, 0, st>>>(sa);
+      PTY_LAUNCH_CHECK("k_scalar_grad", 8);
+    }
+    if (pb.B == 0 && !pb.accumulate) {
+      if ((gm & PTY_GRAD_DZ) && pb.g_dz && cudaMemsetAsync(pb.g_dz, 0, sizeof(float), st) != cudaSuccess)
+        return memset_failed();
+      if ((gm & PTY_GRAD_TILT) && pb.g_tilt && pb.global_tilt &&
+          cudaMemsetAsync(pb.g_tilt, 0, 2 * sizeof(float), st) != cudaSuccess)
+        return memset_failed();
     }
     return PTY_OK;
   }
