@@ -12,6 +12,7 @@
 //                                first transposed to pixel-contiguous rows (chunks of at most 2^18
 //                                pixels), then one plain GEMM per chunk, split over pixels with
 //                                float atomics
+// All of them run through k_gemm_ws (gemm_ws.cuh) with weights, dz and im2col transposes kept as tile images.
 // Layer 6 (upsampling x4, 2 output channels) would waste 126 of 128 GEMM columns, so it runs on the
 // CUDA cores: nearest upsampling makes every output pixel read, for each tap, one low-resolution
 // pixel, so the per-tap channel sums P[p][tap][o] = sum_c W[o][tap][c] a5[p][c] are formed once per
@@ -23,8 +24,7 @@
 #include <stdint.h>
 #include <string.h>
 
-#include "gemm_mma.cuh"
-#include "gemm_tc.cuh"
+#include "gemm_ws.cuh"
 #include "pty_cnn.h"
 #include "pty_internal.h"
 
@@ -58,6 +58,7 @@ struct Plan {
   size_t status, wp[kLayers], wt[kLayers], w6, act[kLayers], dz[kLayers + 1], p6, dp6, du5, lpart, colt, dzt,
       total;
   int pchunk[kLayers];  // pixels per weight-gradient chunk (multiple of 64)
+  size_t colt_elems;    // elements of colt
 };
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -112,6 +113,7 @@ static bool make_plan(int S, int B, Plan* pl) {
     colt = colt > (size_t)9 * kNet[l].ic * p.pchunk[l] ? colt : (size_t)9 * kNet[l].ic * p.pchunk[l];
     dzt = dzt > (size_t)kNet[l].oc * p.pchunk[l] ? dzt : (size_t)kNet[l].oc * p.pchunk[l];
   }
+  p.colt_elems = colt;
   p.colt = take(sizeof(bf16) * colt);
   p.dzt = take(sizeof(bf16) * dzt);
   p.total = off;
@@ -131,12 +133,19 @@ size_t param_count() {
 // ---------------------------------------------------------------------------------------------
 struct PackArgs {
   const float* params;
-  bf16* wp[5];  // [OC][kp]
-  bf16* wt[5];  // [IC][ktp] (layers 2..5)
+  bf16* wp[5];  // tile image [OC][kp]
+  bf16* wt[5];  // tile image [IC][ktp] (layers 2..5)
   float* w6;    // [18][256]: row tap * 2 + o, bf16-rounded
   size_t woff[kLayers];
   int kp[kLayers], ktp[kLayers], ic[kLayers], oc[kLayers];
 };
+
+// (row, k) of element e of a tile image of `rows` rows
+__device__ __forceinline__ void image_element(int e, int rows, int* row, int* k) {
+  const int kb = e / (rows * 64), r = e - kb * rows * 64;
+  *row = (r >> 9) * 8 + ((r >> 3) & 7);
+  *k = kb * 64 + ((r >> 6) & 7) * 8 + (r & 7);
+}
 
 __global__ void k_pack(PackArgs a) {
   // segments: wp of layers 0..4, wt of layers 1..4, w6
@@ -153,11 +162,13 @@ __global__ void k_pack(PackArgs a) {
     while (e >= seg[q]) e -= seg[q++];
     if (q < 5) {  // forward operand of layer q: W[oc][k], k = (ky, kx, ic)
       const int l = q, K9 = 9 * a.ic[l];
-      const int oc = (int)(e / a.kp[l]), k = (int)(e % a.kp[l]);
+      int oc, k;
+      image_element((int)e, a.oc[l], &oc, &k);
       a.wp[l][e] = __float2bfloat16_rn(k < K9 ? a.params[a.woff[l] + (size_t)oc * K9 + k] : 0.f);
     } else if (q < 9) {  // dgrad operand of layer l: Wt[ic][k'] = W[oc][tap][ic], k' = tap * OC + oc
       const int l = q - 4, IC = a.ic[l], OC = a.oc[l];
-      const int ic = (int)(e / a.ktp[l]), kk = (int)(e % a.ktp[l]);
+      int ic, kk;
+      image_element((int)e, a.ic[l], &ic, &kk);
       float w = 0.f;
       if (kk < 9 * OC) {
         const int tap = kk / OC, oc = kk % OC;
@@ -184,178 +195,241 @@ __device__ __forceinline__ bf16 input_value(const float* I, float s_in, int S, i
   return __float2bfloat16_rn(s_in * log1pf(__ldg(I + ((size_t)b * S + y) * S + x)));
 }
 
-// Forward of layer 1: rows = output pixels, k = tap (9 of 32 used); values from the FP32 patterns.
-struct InputIm2col {
-  const float* I;
-  float s_in;
-  int S, B, hout;
-  __device__ __forceinline__ uint4 operator()(int m, int k) const {
-    Pack8 r;
-    r.u = make_uint4(0u, 0u, 0u, 0u);
-    if (m >= B * hout * hout || k >= 9) return r.u;
-    const int b = m / (hout * hout), rem = m % (hout * hout), oy = rem / hout, ox = rem % hout;
+// Layer 1's rows: x16[pixel][16] = the nine taps of bf16(s_in log(1 + I)) (zeros outside) and seven zeros, written once
+// so that the GEMM gathers 32 contiguous bytes a row.  Rows p0 .. p0 + n - 1; one thread per row.
+__global__ void __launch_bounds__(256) k_input_rows(const float* __restrict__ I, float s_in, bf16* __restrict__ x16, int S,
+                                                    int hout, size_t p0, size_t n) {
+  const size_t i = blockIdx.x * (size_t)256 + threadIdx.x;
+  if (i >= n) return;
+  const size_t m = p0 + i, hw = (size_t)hout * hout;
+  const int b = (int)(m / hw), rem = (int)(m % hw), oy = rem / hout, ox = rem % hout;
+  Pack8 r[2];
+  r[0].u = r[1].u = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const int tap = k + e;
-      if (tap < 9) {
-        const int y = 2 * oy + tap / 3 - 1, x = 2 * ox + tap % 3 - 1;
-        if (y >= 0 && y < S && x >= 0 && x < S) r.h[e] = input_value(I, s_in, S, b, y, x);
-      }
-    }
-    return r.u;
+  for (int tap = 0; tap < 9; ++tap) {
+    const int y = 2 * oy + tap / 3 - 1, x = 2 * ox + tap % 3 - 1;
+    if (y >= 0 && y < S && x >= 0 && x < S) r[tap / 8].h[tap % 8] = input_value(I, s_in, S, b, y, x);
   }
+  uint4* o = reinterpret_cast<uint4*>(x16 + 16 * i);
+  o[0] = r[0].u;
+  o[1] = r[1].u;
+}
+struct InputRows {
+  static constexpr bool kGather = true;
+  const bf16* x16;
+  int rows;
+  struct K {
+    int tap, off;
+  };
+  __device__ __forceinline__ const bf16* any() const { return x16; }
+  __device__ __forceinline__ int kb_next(int, int kb) const { return kb; }
+  __device__ __forceinline__ GatherRow row(int m) const { return GatherRow{x16 + (size_t)m * 16, m < rows ? 1u : 0u, 0u}; }
+  __device__ __forceinline__ K kpos(int k) const { return K{0, k}; }
+  __device__ __forceinline__ int offset(const GatherRow&, const K& k) const { return k.off; }
 };
 
-// Forward of layers 2..5: 8 channels of one tap of the (upsampled) input, 16-byte loads.
+// Forward of layers 2..5: rows = output pixels, 8 channels of one tap of the (upsampled) input per chunk.  A tap's
+// distance from tap 0 is the same for every row, or with upsampling depends on the parities of the row's pixel
+// (bits 16, 17 of its mask).
+template <int UP>
 struct Im2col {
+  static constexpr bool kGather = true;
   const bf16* a;  // [B][hin][hin][ic]
-  int B, hin, hu, hout, ic, stride, up;
-  __device__ __forceinline__ uint4 operator()(int m, int k) const {
-    if (m >= B * hout * hout || k >= 9 * ic) return make_uint4(0u, 0u, 0u, 0u);
-    const int b = m / (hout * hout), rem = m % (hout * hout), oy = rem / hout, ox = rem % hout;
-    const int tap = k / ic, c0 = k - tap * ic;
-    const int uy = stride * oy + tap / 3 - 1, ux = stride * ox + tap % 3 - 1;
-    if (uy < 0 || uy >= hu || ux < 0 || ux >= hu) return make_uint4(0u, 0u, 0u, 0u);
-    return __ldg(reinterpret_cast<const uint4*>(a + (((size_t)b * hin + uy / up) * hin + ux / up) * ic + c0));
-  }
-  // cursor: the output pixel decoded once, (tap, channel) stepped through K
-  struct Cursor {
-    const bf16* img;  // sample b of the input, or nullptr past the last row
-    int y0, x0;       // stride * (oy, ox) - 1 on the upsampled grid
-    int ky, kx, c0;
+  int B, hin, hu, hout, ic, stride;
+  struct K {
+    int tap, y[UP], x[UP];  // elements, by the parity of the pixel; x holds the channel too
   };
-  __device__ __forceinline__ Cursor cursor(int m, int k) const {
-    Cursor c;
-    c.img = nullptr;
-    c.y0 = c.x0 = 0;
-    if (m < B * hout * hout) {
-      const int b = m / (hout * hout), rem = m % (hout * hout);
-      c.img = a + (size_t)b * hin * hin * ic;
-      c.y0 = stride * (rem / hout) - 1;
-      c.x0 = stride * (rem % hout) - 1;
-    }
-    const int tap = k / ic;
-    c.ky = tap / 3;
-    c.kx = tap % 3;
-    c.c0 = k - tap * ic;
-    return c;
+  __device__ __forceinline__ const bf16* any() const { return a; }
+  __device__ __forceinline__ int kb_next(int, int kb) const { return kb; }
+  __device__ __forceinline__ GatherRow row(int m) const {
+    if (m >= B * hout * hout) return GatherRow{a, 0u, 0u};
+    const int b = m / (hout * hout), rem = m - b * hout * hout, oy = rem / hout;
+    const int y0 = stride * oy - 1, x0 = stride * (rem - oy * hout) - 1;
+    unsigned mask = 0;
+#pragma unroll
+    for (int t = 0; t < 9; ++t)
+      if ((unsigned)(y0 + t / 3) < (unsigned)hu && (unsigned)(x0 + t % 3) < (unsigned)hu) mask |= 1u << t;
+    if (UP == 2) mask |= (unsigned)(y0 & 1) << 16 | (unsigned)(x0 & 1) << 17;
+    const long long pix = (long long)(b * hin + (y0 >> (UP - 1))) * hin + (x0 >> (UP - 1));
+    return GatherRow{a + pix * ic, mask, 0u};
   }
-  __device__ __forceinline__ uint4 load(const Cursor& c) const {
-    const int uy = c.y0 + c.ky, ux = c.x0 + c.kx;
-    if (!c.img || c.ky > 2 || uy < 0 || uy >= hu || ux < 0 || ux >= hu) return make_uint4(0u, 0u, 0u, 0u);
-    const int sh = up == 2 ? 1 : 0;  // up is 1 or 2 for the layers that gather this way
-    return __ldg(reinterpret_cast<const uint4*>(c.img + ((size_t)(uy >> sh) * hin + (ux >> sh)) * ic + c.c0));
-  }
-  __device__ __forceinline__ void advance(Cursor& c, int dk) const {
-    c.c0 += dk;
-    while (c.c0 >= ic) {
-      c.c0 -= ic;
-      if (++c.kx == 3) {
-        c.kx = 0;
-        ++c.ky;
-      }
+  __device__ __forceinline__ K kpos(int k) const {
+    K r;
+    r.tap = k / ic;
+    const int ky = r.tap / 3, kx = r.tap - 3 * ky;
+#pragma unroll
+    for (int p = 0; p < UP; ++p) {
+      r.y[p] = ((p + ky) >> (UP - 1)) * hin * ic;
+      r.x[p] = ((p + kx) >> (UP - 1)) * ic + k - r.tap * ic;
     }
+    return r;
+  }
+  __device__ __forceinline__ int offset(const GatherRow& r, const K& k) const {
+    if constexpr (UP == 1) return k.y[0] + k.x[0];
+    else return ((r.m >> 16 & 1) ? k.y[1] : k.y[0]) + ((r.m >> 17 & 1) ? k.x[1] : k.x[0]);
   }
 };
 
-// Input gradient of layers 2..5: rows = pixels of the upsampled input grid, k' = (tap, oc); the
-// output pixel that reads (uy, ux) through tap (ky, kx) is ((uy + 1 - ky) / s, (ux + 1 - kx) / s).
+// Rows of an input gradient: the pixels of the (upsampled) input grid.  With stride 2 a pixel (uy, ux) is reached
+// only by the taps with ky = uy + 1 and kx = ux + 1 (mod 2), one to four of nine, so the pixels are taken in four
+// classes by their parities, whole row tiles each, and a tile skips the K blocks of the other taps: those
+// would add exact zeros (about 2.6 of 9 of the blocks are left).
+struct GradRows {
+  int B, hu, stride, ctiles;  // ctiles: row tiles of a class
+  __host__ __device__ GradRows(int B_, int hu_, int stride_) : B(B_), hu(hu_), stride(stride_) {
+    const int h = hu / stride;
+    ctiles = (B * h * h + 127) / 128;
+  }
+  int row_tiles() const { return ctiles * stride * stride; }
+  __device__ __forceinline__ int tile_class(int tile) const { return stride == 2 ? tile / ctiles : 0; }
+  // class, sample and place (in units of the stride) of row m; false past the end of its class
+  __device__ __forceinline__ bool pixel(int m, int* cls, int* b, int* y, int* x) const {
+    *cls = tile_class(m >> 7);
+    const int i = m - *cls * ctiles * 128, h = hu / stride;
+    if (i >= B * h * h) return false;
+    *b = i / (h * h);
+    const int rem = i - *b * h * h;
+    *y = rem / h;
+    *x = rem - *y * h;
+    return true;
+  }
+};
+// Input gradient of layers 2..5: k' = (tap, oc); the output pixel that reads (uy, ux) through tap (ky, kx) is
+// ((uy + 1 - ky) / s, (ux + 1 - kx) / s).
 struct DgradGather {
+  static constexpr bool kGather = true;
   const bf16* dz;  // [B][hout][hout][oc]
-  int B, hu, hout, oc, stride;
-  __device__ __forceinline__ uint4 operator()(int m, int k) const {
-    if (m >= B * hu * hu || k >= 9 * oc) return make_uint4(0u, 0u, 0u, 0u);
-    const int b = m / (hu * hu), rem = m % (hu * hu), uy = rem / hu, ux = rem % hu;
-    const int tap = k / oc, o0 = k - tap * oc;
-    const int ty = uy + 1 - tap / 3, tx = ux + 1 - tap % 3;
-    if (ty < 0 || tx < 0 || ty % stride || tx % stride) return make_uint4(0u, 0u, 0u, 0u);
-    const int oy = ty / stride, ox = tx / stride;
-    if (oy >= hout || ox >= hout) return make_uint4(0u, 0u, 0u, 0u);
-    return __ldg(reinterpret_cast<const uint4*>(dz + (((size_t)b * hout + oy) * hout + ox) * oc + o0));
-  }
-  struct Cursor {
-    const bf16* img;  // sample b of dz, or nullptr past the last row
-    int y1, x1;       // (uy + 1, ux + 1)
-    int ky, kx, o0;
-  };
-  __device__ __forceinline__ Cursor cursor(int m, int k) const {
-    Cursor c;
-    c.img = nullptr;
-    c.y1 = c.x1 = 0;
-    if (m < B * hu * hu) {
-      const int b = m / (hu * hu), rem = m % (hu * hu);
-      c.img = dz + (size_t)b * hout * hout * oc;
-      c.y1 = rem / hu + 1;
-      c.x1 = rem % hu + 1;
+  GradRows g;
+  int hout, oc;
+  unsigned long long blocks[4];  // K blocks with a tap of the class (bit kb; at most 54 blocks)
+  DgradGather(const bf16* dz_, const GradRows& g_, int hout_, int oc_, int kb_all) : dz(dz_), g(g_), hout(hout_), oc(oc_) {
+    for (int c = 0; c < 4; ++c) {
+      blocks[c] = 0;
+      for (int kb = 0; kb < kb_all; ++kb)
+        for (int t = kb * kWsBlock / oc; t <= (kb * kWsBlock + kWsBlock - 1) / oc && t < 9; ++t)
+          if (g.stride == 1 || (!(((c >> 1) + 1 - t / 3) & 1) && !(((c & 1) + 1 - t % 3) & 1))) blocks[c] |= 1ull << kb;
     }
-    const int tap = k / oc;
-    c.ky = tap / 3;
-    c.kx = tap % 3;
-    c.o0 = k - tap * oc;
-    return c;
   }
-  __device__ __forceinline__ uint4 load(const Cursor& c) const {
-    const int ty = c.y1 - c.ky, tx = c.x1 - c.kx;
-    const int sm = stride - 1, sh = stride == 2 ? 1 : 0;  // stride is 1 or 2
-    if (!c.img || c.ky > 2 || ty < 0 || tx < 0 || ((ty | tx) & sm)) return make_uint4(0u, 0u, 0u, 0u);
-    const int oy = ty >> sh, ox = tx >> sh;
-    if (oy >= hout || ox >= hout) return make_uint4(0u, 0u, 0u, 0u);
-    return __ldg(reinterpret_cast<const uint4*>(c.img + ((size_t)oy * hout + ox) * oc + c.o0));
+  struct K {
+    int tap, y, x;  // (ky, kx) for stride 2; y the whole offset for stride 1
+  };
+  __device__ __forceinline__ const bf16* any() const { return dz; }
+  __device__ __forceinline__ int kb_next(int tile, int kb) const {
+    if (g.stride == 1) return kb;
+    const int c = g.tile_class(tile);
+    const unsigned long long left = (c == 0 ? blocks[0] : c == 1 ? blocks[1] : c == 2 ? blocks[2] : blocks[3]) >> kb;  // kb <= 54
+    return left ? kb + __ffsll((long long)left) - 1 : 64;
   }
-  __device__ __forceinline__ void advance(Cursor& c, int dk) const {
-    c.o0 += dk;
-    while (c.o0 >= oc) {
-      c.o0 -= oc;
-      if (++c.kx == 3) {
-        c.kx = 0;
-        ++c.ky;
+  __device__ __forceinline__ GatherRow row(int m) const {
+    int cls, b, y, x;
+    if (!g.pixel(m, &cls, &b, &y, &x)) return GatherRow{dz, 0u, 0u};
+    unsigned mask = 0;
+    if (g.stride == 1) {  // tap (ky, kx) reads (y + 1 - ky, x + 1 - kx)
+#pragma unroll
+      for (int t = 0; t < 9; ++t)
+        if ((unsigned)(y + 1 - t / 3) < (unsigned)hout && (unsigned)(x + 1 - t % 3) < (unsigned)hout) mask |= 1u << t;
+    } else {  // the taps of the class: (y + (py + 1 - ky) / 2, ...)
+      const int py = cls >> 1, px = cls & 1;
+#pragma unroll
+      for (int t = 0; t < 9; ++t) {
+        const int dy = py + 1 - t / 3, dx = px + 1 - t % 3;
+        if (!((dy | dx) & 1) && (unsigned)(y + (dy >> 1)) < (unsigned)hout && (unsigned)(x + (dx >> 1)) < (unsigned)hout)
+          mask |= 1u << t;
       }
     }
+    mask |= (unsigned)cls << 16;
+    return GatherRow{dz + ((size_t)(b * hout + y) * hout + x) * oc, mask, 0u};
   }
+  __device__ __forceinline__ K kpos(int k) const {
+    const int tap = k / oc, ky = tap / 3, kx = tap - 3 * ky, o = k - tap * oc;
+    if (g.stride == 1) return K{tap, ((1 - ky) * hout + 1 - kx) * oc + o, 0};
+    return K{tap, ky, (o << 2) | kx};
+  }
+  __device__ __forceinline__ int offset(const GatherRow& r, const K& k) const {
+    if (g.stride == 1) return k.y;
+    const int py = r.m >> 17 & 1, px = r.m >> 16 & 1;
+    return (((py + 1 - k.y) >> 1) * hout + ((px + 1 - (k.x & 3)) >> 1)) * oc + (k.x >> 2);
+  }
+};
+struct ImageLoad {
+  static constexpr bool kGather = false;
+  ImageOperand op;
 };
 
 // ---------------------------------------------------------------------------------------------
 // GEMM epilogues
 // ---------------------------------------------------------------------------------------------
+// epi(row, col, v): eight consecutive columns
 struct FwdEpi {  // a = bf16(relu(z + bias))
   bf16* out;
   const float* bias;
   int rows, oc;
-  __device__ __forceinline__ void operator()(int row, int col, float v0, float v1) const {
-    if (row >= rows || col >= oc) return;
-    v0 = fmaxf(v0 + bias[col], 0.f);
-    v1 = fmaxf(v1 + bias[col + 1], 0.f);
-    *reinterpret_cast<__nv_bfloat162*>(out + (size_t)row * oc + col) = __floats2bfloat162_rn(v0, v1);
+  using Row = int;
+  __device__ __forceinline__ Row prep(int m) const { return m; }
+  __device__ __forceinline__ void operator()(int row, int col, const float* v) const {
+    if (row >= rows) return;
+    Pack8 r;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) r.h[e] = __float2bfloat16_rn(fmaxf(v[e] + __ldg(bias + col + e), 0.f));
+    *reinterpret_cast<uint4*>(out + (size_t)row * oc + col) = r.u;
   }
 };
 struct DgradEpi {  // dz of the layer below = bf16(du * (a > 0)) (no upsampling between)
   bf16* dz;
   const bf16* a;
-  int rows, ic;
-  __device__ __forceinline__ void operator()(int row, int col, float v0, float v1) const {
-    if (row >= rows || col >= ic) return;
+  GradRows g;
+  int ic;
+  using Row = long long;
+  __device__ __forceinline__ Row prep(int m) const {  // its pixel, or -1
+    int cls, b, y, x;
+    if (!g.pixel(m, &cls, &b, &y, &x)) return -1;
+    return ((long long)b * g.hu + g.stride * y + (g.stride == 2 ? cls >> 1 : 0)) * g.hu + g.stride * x +
+           (g.stride == 2 ? cls & 1 : 0);
+  }
+  __device__ __forceinline__ void operator()(Row row, int col, const float* v) const {
+    if (row < 0) return;
     const size_t e = (size_t)row * ic + col;
-    const __nv_bfloat162 av = *reinterpret_cast<const __nv_bfloat162*>(a + e);
-    v0 = __low2float(av) > 0.f ? v0 : 0.f;
-    v1 = __high2float(av) > 0.f ? v1 : 0.f;
-    *reinterpret_cast<__nv_bfloat162*>(dz + e) = __floats2bfloat162_rn(v0, v1);
+    Pack8 av, r;
+    av.u = __ldg(reinterpret_cast<const uint4*>(a + e));
+#pragma unroll
+    for (int k = 0; k < 8; ++k) r.h[k] = __float2bfloat16_rn(__bfloat162float(av.h[k]) > 0.f ? v[k] : 0.f);
+    *reinterpret_cast<uint4*>(dz + e) = r.u;
   }
 };
 struct StoreEpi {  // FP32 store (gradient on the upsampled grid)
   float* out;
   int rows, cols;
-  __device__ __forceinline__ void operator()(int row, int col, float v0, float v1) const {
-    if (row >= rows || col >= cols) return;
-    *reinterpret_cast<float2*>(out + (size_t)row * cols + col) = make_float2(v0, v1);
+  using Row = int;
+  __device__ __forceinline__ Row prep(int m) const { return m; }
+  __device__ __forceinline__ void operator()(int row, int col, const float* v) const {
+    if (row >= rows) return;
+    float4* o = reinterpret_cast<float4*>(out + (size_t)row * cols + col);
+    o[0] = make_float4(v[0], v[1], v[2], v[3]);
+    o[1] = make_float4(v[4], v[5], v[6], v[7]);
   }
 };
-struct WgradEpi {  // split-K partial sums of dW[oc][k]
+struct WgradImageEpi {  // split-K partial sums of dW[oc][k]; k9 a multiple of 8
   float* g;
   int oc, k9;
-  __device__ __forceinline__ void operator()(int row, int col, float v0, float v1) const {
+  using Row = int;
+  __device__ __forceinline__ Row prep(int m) const { return m; }
+  __device__ __forceinline__ void operator()(int row, int col, const float* v) const {
+    if (row >= oc || col >= k9) return;
+    float4* o = reinterpret_cast<float4*>(g + (size_t)row * k9 + col);
+    atomicAdd(o, make_float4(v[0], v[1], v[2], v[3]));
+    atomicAdd(o + 1, make_float4(v[4], v[5], v[6], v[7]));
+  }
+};
+struct WgradEpi {  // the same for layer 1 (nine columns)
+  float* g;
+  int oc, k9;
+  using Row = int;
+  __device__ __forceinline__ Row prep(int m) const { return m; }
+  __device__ __forceinline__ void operator()(int row, int col, const float* v) const {
     if (row >= oc) return;
-    if (col < k9) atomicAdd(g + (size_t)row * k9 + col, v0);
-    if (col + 1 < k9) atomicAdd(g + (size_t)row * k9 + col + 1, v1);
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      if (col + e < k9) atomicAdd(g + (size_t)row * k9 + col + e, v[e]);
   }
 };
 
@@ -363,34 +437,33 @@ struct WgradEpi {  // split-K partial sums of dW[oc][k]
 // ---------------------------------------------------------------------------------------------
 // Layer 6 on the CUDA cores
 // ---------------------------------------------------------------------------------------------
-// P[p][j] = sum_c w6[j][c] a5[p][c]: one warp per low-resolution pixel, 8 channels per lane.
-__global__ void __launch_bounds__(256) k_l6_sums(const bf16* __restrict__ a5, const float* __restrict__ w6,
+// P[p][j] = sum_c w6[j][c] a5[p][c]: one warp per low-resolution pixel, 8 channels per lane; a warp keeps its lanes'
+// weights in registers over all its pixels (loaded through shared memory by every 8 pixels: 97 us on 65536).
+__global__ void __launch_bounds__(128) k_l6_sums(const bf16* __restrict__ a5, const float* __restrict__ w6,
                                                  float* __restrict__ P, int npix) {
-  __shared__ float w[kTaps6 * kC6];
-  for (int i = threadIdx.x; i < kTaps6 * kC6; i += blockDim.x) w[i] = w6[i];
-  __syncthreads();
   const int lane = threadIdx.x & 31;
-  const int p = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (p >= npix) return;
-  Pack8 v;
-  v.u = __ldg(reinterpret_cast<const uint4*>(a5 + (size_t)p * kC6 + lane * 8));
-  float x[8];
-#pragma unroll
-  for (int e = 0; e < 8; ++e) x[e] = __bfloat162float(v.h[e]);
-  float acc[kTaps6];
-#pragma unroll
-  for (int j = 0; j < kTaps6; ++j) {
-    float t = 0.f;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) t = fmaf(w[j * kC6 + lane * 8 + e], x[e], t);
-    acc[j] = t;
-  }
+  float w[kTaps6][8];
 #pragma unroll
   for (int j = 0; j < kTaps6; ++j)
-    for (int o = 16; o > 0; o >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
-  if (lane == 0) {
 #pragma unroll
-    for (int j = 0; j < kTaps6; ++j) P[(size_t)p * kTaps6 + j] = acc[j];
+    for (int e = 0; e < 8; ++e) w[j][e] = __ldg(w6 + j * kC6 + lane * 8 + e);
+  for (int p = blockIdx.x * 4 + (threadIdx.x >> 5); p < npix; p += gridDim.x * 4) {
+    Pack8 v;
+    v.u = __ldg(reinterpret_cast<const uint4*>(a5 + (size_t)p * kC6 + lane * 8));
+    float x[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) x[e] = __bfloat162float(v.h[e]);
+    float mine = 0.f;
+#pragma unroll
+    for (int j = 0; j < kTaps6; ++j) {
+      float t = 0.f;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) t = fmaf(w[j][e], x[e], t);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane == j) mine = t;
+    }
+    if (lane < kTaps6) P[(size_t)p * kTaps6 + lane] = mine;
   }
 }
 
@@ -465,30 +538,44 @@ __global__ void k_l6_dsums(const bf16* __restrict__ dz6, float* __restrict__ dP,
   }
 }
 
-// dz5[p][c] = bf16((a5[p][c] > 0) sum_j dP[p][j] w6[j][c]).
-__global__ void __launch_bounds__(256) k_l6_dgrad(const float* __restrict__ dP, const float* __restrict__ w6,
-                                                  const bf16* __restrict__ a5, bf16* __restrict__ dz5, int npix) {
-  const int p = blockIdx.x, c = threadIdx.x;  // blockDim = 256 channels
-  if (p >= npix) return;
-  __shared__ float d[kTaps6];
-  if (c < kTaps6) d[c] = dP[(size_t)p * kTaps6 + c];
-  __syncthreads();
-  float acc = 0.f;
+// dz5[p][c] = bf16((a5[p][c] > 0) sum_j dP[p][j] w6[j][c]) and dW6[o][tap][c] += sum over the CTA's pixels of dP[p][tap 2 + o]
+// a5[p][c]: thread c keeps its channel's weights and sums in registers, eight pixels' operands in flight (a
+// CTA per pixel, and a pass over a5 per tap and output: 64 + 131 us on 65536 pixels).
+__global__ void __launch_bounds__(kC6) k_l6_grad(const float* __restrict__ dP, const float* __restrict__ w6,
+                                                 const bf16* __restrict__ a5, bf16* __restrict__ dz5, float* __restrict__ gW6,
+                                                 int npix) {
+  constexpr int U = 8;
+  __shared__ float d[U * kTaps6];
+  const int c = threadIdx.x;
+  float w[kTaps6], g[kTaps6];
 #pragma unroll
-  for (int j = 0; j < kTaps6; ++j) acc = fmaf(d[j], __ldg(w6 + j * kC6 + c), acc);
-  const size_t e = (size_t)p * kC6 + c;
-  dz5[e] = __float2bfloat16_rn(__bfloat162float(a5[e]) > 0.f ? acc : 0.f);
-}
-
-// dW6[o][tap][c] += sum over a chunk of pixels of dP[p][tap * 2 + o] a5[p][c].
-__global__ void __launch_bounds__(256) k_l6_wgrad(const float* __restrict__ dP, const bf16* __restrict__ a5,
-                                                  float* __restrict__ gW6, int npix, int chunk) {
-  const int j = blockIdx.y, c = threadIdx.x, p0 = blockIdx.x * chunk;
-  const int p1 = p0 + chunk < npix ? p0 + chunk : npix;
-  float acc = 0.f;
-  for (int p = p0; p < p1; ++p) acc = fmaf(__ldg(dP + (size_t)p * kTaps6 + j), __bfloat162float(a5[(size_t)p * kC6 + c]), acc);
-  const int tap = j / kOut, o = j % kOut;
-  atomicAdd(gW6 + ((size_t)o * 9 + tap) * kC6 + c, acc);
+  for (int j = 0; j < kTaps6; ++j) {
+    w[j] = __ldg(w6 + j * kC6 + c);
+    g[j] = 0.f;
+  }
+  for (int p0 = blockIdx.x * U; p0 < npix; p0 += gridDim.x * U) {
+    const int n = min(U, npix - p0);
+    __syncthreads();
+    if (c < n * kTaps6) d[c] = dP[(size_t)p0 * kTaps6 + c];
+    float a[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) a[u] = u < n ? __bfloat162float(a5[(size_t)(p0 + u) * kC6 + c]) : 0.f;
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (u >= n) break;
+      float acc = 0.f;
+#pragma unroll
+      for (int j = 0; j < kTaps6; ++j) {
+        const float dj = d[u * kTaps6 + j];
+        acc = fmaf(dj, w[j], acc);
+        g[j] = fmaf(dj, a[u], g[j]);
+      }
+      dz5[(size_t)(p0 + u) * kC6 + c] = __float2bfloat16_rn(a[u] > 0.f ? acc : 0.f);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < kTaps6; ++j) atomicAdd(gW6 + ((size_t)(j % kOut) * 9 + j / kOut) * kC6 + c, g[j]);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -505,19 +592,34 @@ __global__ void k_bias_grad(const bf16* __restrict__ dz, float* __restrict__ gb,
   }
 }
 
-// dz[b][y][x][c] = bf16((a > 0) sum of the f x f block of du on the upsampled grid).
-__global__ void k_upsample_grad(const float* __restrict__ du, const bf16* __restrict__ a, bf16* __restrict__ dz, int B,
-                                int h, int C, int f) {
-  const size_t n = (size_t)B * h * h * C;
+// dz[b][y][x][c] = bf16((a > 0) sum of the f x f block of du on the upsampled grid), four channels a thread.
+__global__ void __launch_bounds__(256) k_upsample_grad(const float* __restrict__ du, const bf16* __restrict__ a,
+                                                       bf16* __restrict__ dz, int B, int h, int C, int f) {
+  const size_t n = (size_t)B * h * h * C / 4;
   const int hu = h * f;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const int c = (int)(i % C);
-    const size_t px = i / C;
+  for (size_t i = blockIdx.x * (size_t)256 + threadIdx.x; i < n; i += (size_t)gridDim.x * 256) {
+    const int c = 4 * (int)(i % (C / 4));
+    const size_t px = i / (C / 4);
     const int x = (int)(px % h), y = (int)((px / h) % h), b = (int)(px / ((size_t)h * h));
-    float acc = 0.f;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int dy = 0; dy < f; ++dy)
-      for (int dx = 0; dx < f; ++dx) acc += du[(((size_t)b * hu + f * y + dy) * hu + f * x + dx) * C + c];
-    dz[i] = __float2bfloat16_rn(__bfloat162float(a[i]) > 0.f ? acc : 0.f);
+      for (int dx = 0; dx < f; ++dx) {
+        const float4 v = *reinterpret_cast<const float4*>(du + (((size_t)b * hu + f * y + dy) * hu + f * x + dx) * C + c);
+        acc.x += v.x;
+        acc.y += v.y;
+        acc.z += v.z;
+        acc.w += v.w;
+      }
+    union {
+      uint2 u;
+      bf16 e[4];
+    } av, r;
+    av.u = *reinterpret_cast<const uint2*>(a + px * C + c);
+    r.e[0] = __float2bfloat16_rn(__bfloat162float(av.e[0]) > 0.f ? acc.x : 0.f);
+    r.e[1] = __float2bfloat16_rn(__bfloat162float(av.e[1]) > 0.f ? acc.y : 0.f);
+    r.e[2] = __float2bfloat16_rn(__bfloat162float(av.e[2]) > 0.f ? acc.z : 0.f);
+    r.e[3] = __float2bfloat16_rn(__bfloat162float(av.e[3]) > 0.f ? acc.w : 0.f);
+    *reinterpret_cast<uint2*>(dz + px * C + c) = r.u;
   }
 }
 
@@ -598,16 +700,39 @@ __global__ void k_stitch_finish(int Nz, int H, int W, const float* __restrict__ 
 // ---------------------------------------------------------------------------------------------
 // Weight-gradient operands with pixel-contiguous rows
 // ---------------------------------------------------------------------------------------------
-// colT[k][m - p0] = im2col[m][k] for k = (tap, ic) < 9 IC and output pixels m in [p0, p0 + P); zero
-// past the last pixel (layers 2..5, ic a multiple of 8).  A thread takes one pixel and 8 channels:
-// per tap one 16-byte load and 8 stores into 8 rows; consecutive threads take consecutive pixels, so
-// every row is written 64 bytes per warp at a time.
-__global__ void k_im2col_t(const bf16* __restrict__ a, bf16* __restrict__ colt, int B, int hin, int hu, int hout,
-                           int ic, int stride, int up, int p0, int P) {
-  const int hw = hout * hout, pixels = B * hw, groups = ic / 8;
-  const size_t n = (size_t)groups * P;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const int mm = (int)(i % P), c0 = 8 * (int)(i / P), m = p0 + mm;
+// Transpose of 8 x 8 16-bit values over eight consecutive lanes: lane p's r[i] holds values 2 i, 2 i + 1 of row p; afterwards
+// of column p.
+__device__ __forceinline__ void transpose8(uint32_t (&r)[4], int lane) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t o = __shfl_xor_sync(0xffffffffu, r[i], 1);
+    r[i] = (lane & 1) ? __byte_perm(o, r[i], 0x7632) : __byte_perm(r[i], o, 0x5410);
+  }
+#pragma unroll
+  for (int i = 0; i < 4; i += 2) {
+    const uint32_t o = __shfl_xor_sync(0xffffffffu, (lane & 2) ? r[i] : r[i + 1], 2);
+    if (lane & 2) r[i] = o;
+    else r[i + 1] = o;
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const uint32_t o = __shfl_xor_sync(0xffffffffu, (lane & 4) ? r[i] : r[i + 2], 4);
+    if (lane & 4) r[i] = o;
+    else r[i + 2] = o;
+  }
+}
+
+// Tile image of colT[k][m - p0] = im2col[m][k] for k = (tap, ic) < 9 IC and output pixels m in [p0, p0 + P); zero past the
+// last pixel (layers 2..5, ic a multiple of 16).  A warp takes 16 pixels by two groups of 8 channels: per tap each
+// lane loads its pixel's 16 bytes, eight lanes transpose 8 pixels x 8 channels, and every store is one core
+// matrix row, 128 contiguous bytes per eight lanes.
+__global__ void __launch_bounds__(256) k_im2col_t(const bf16* __restrict__ a, bf16* __restrict__ colt, int B, int hin, int hu,
+                                                  int hout, int ic, int stride, int up, int p0, int P) {
+  const int hw = hout * hout, pixels = B * hw, pairs = ic / 16, k9 = 9 * ic, lane = threadIdx.x & 31;
+  const size_t warps = (size_t)pairs * (P / 16), step = (size_t)gridDim.x * 8;
+  const int sh = up == 2 ? 1 : 0;
+  for (size_t w = blockIdx.x * (size_t)8 + (threadIdx.x >> 5); w < warps; w += step) {
+    const int mm = (int)(w / pairs) * 16 + (lane & 15), c0 = (int)(w % pairs) * 16 + 8 * (lane >> 4), m = p0 + mm;
     int b = 0, y0 = -1 << 20, x0 = -1 << 20;
     if (m < pixels) {
       b = m / hw;
@@ -616,66 +741,71 @@ __global__ void k_im2col_t(const bf16* __restrict__ a, bf16* __restrict__ colt, 
       x0 = stride * (rem % hout) - 1;
     }
     const bf16* img = a + (size_t)b * hin * hin * ic + c0;
-#pragma unroll 1
+#pragma unroll
     for (int tap = 0; tap < 9; ++tap) {
       const int uy = y0 + tap / 3, ux = x0 + tap % 3;
-      union {
-        uint4 u;
-        bf16 h[8];
-      } v;
-      v.u = make_uint4(0u, 0u, 0u, 0u);
+      uint4 v = make_uint4(0u, 0u, 0u, 0u);
       if (uy >= 0 && uy < hu && ux >= 0 && ux < hu)
-        v.u = __ldg(reinterpret_cast<const uint4*>(img + ((size_t)(uy / up) * hin + ux / up) * ic));
-      bf16* row = colt + ((size_t)tap * ic + c0) * P + mm;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) row[(size_t)e * P] = v.h[e];
+        v = __ldg(reinterpret_cast<const uint4*>(img + ((size_t)(uy >> sh) * hin + (ux >> sh)) * ic));
+      uint32_t r[4] = {v.x, v.y, v.z, v.w};
+      transpose8(r, lane);
+      // this lane now holds channel c0 + lane % 8 of the eight pixels from mm & ~7
+      *reinterpret_cast<uint4*>(colt + image_index(tap * ic + c0 + (lane & 7), (size_t)(mm & ~7), k9)) =
+          make_uint4(r[0], r[1], r[2], r[3]);
     }
   }
 }
 
-// Layer 1 (one channel from the patterns): colT[tap][m - p0], threads along m.
-__global__ void k_im2col_t1(const float* __restrict__ I, float s_in, bf16* __restrict__ colt, int B, int S, int hout,
-                            int p0, int P) {
-  const size_t n = (size_t)9 * P;
-  const int hw = hout * hout, pixels = B * hw;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const int m = p0 + (int)(i % P), tap = (int)(i / P);
-    bf16 v = __float2bfloat16_rn(0.f);
+// Layer 1 (one channel from the patterns): tile image of sixteen rows, taps 0..8 and zeros, of pixels [p0, p0 + P).
+__global__ void __launch_bounds__(256) k_im2col_t1(const float* __restrict__ I, float s_in, bf16* __restrict__ colt, int B,
+                                                   int S, int hout, int p0, int P) {
+  const int hw = hout * hout, pixels = B * hw, lane = threadIdx.x & 31;
+  for (int mm = blockIdx.x * 256 + threadIdx.x; mm < P; mm += gridDim.x * 256) {  // P a multiple of 64: whole warps
+    const int m = p0 + mm;
+    Pack8 lo, hi;
+    lo.u = hi.u = make_uint4(0u, 0u, 0u, 0u);
     if (m < pixels) {
       const int b = m / hw, rem = m % hw, oy = rem / hout, ox = rem % hout;
-      const int y = 2 * oy + tap / 3 - 1, x = 2 * ox + tap % 3 - 1;
-      if (y >= 0 && y < S && x >= 0 && x < S) v = input_value(I, s_in, S, b, y, x);
+#pragma unroll
+      for (int tap = 0; tap < 9; ++tap) {
+        const int y = 2 * oy + tap / 3 - 1, x = 2 * ox + tap % 3 - 1;
+        if (y >= 0 && y < S && x >= 0 && x < S) (tap < 8 ? lo : hi).h[tap & 7] = input_value(I, s_in, S, b, y, x);
+      }
     }
-    colt[i] = v;
+    uint32_t r[4] = {lo.u.x, lo.u.y, lo.u.z, lo.u.w}, t[4] = {hi.u.x, 0u, 0u, 0u};
+    transpose8(r, lane);
+    transpose8(t, lane);
+    bf16* o = colt + image_index(lane & 7, (size_t)(mm & ~7), 16);
+    *reinterpret_cast<uint4*>(o) = make_uint4(r[0], r[1], r[2], r[3]);
+    *reinterpret_cast<uint4*>(o + 512) = make_uint4(t[0], t[1], t[2], t[3]);  // rows 8..15
   }
 }
 
-// dzT[c][m - p0] = dz[m][c] for m in [p0, p0 + P) (zero past the last pixel), 32 x 32 tiles through
-// shared memory, and the bias gradient: gb[c] += the tile's sum over its pixels.
-__global__ void k_dz_t(const bf16* __restrict__ dz, bf16* __restrict__ dzt, float* __restrict__ gb, int pixels, int C,
-                       int p0, int P) {
-  __shared__ bf16 tile[32][34];
-  __shared__ float colsum[8][32];
-  const int mt = blockIdx.x * 32, ct = blockIdx.y * 32;
-  const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
-  float acc = 0.f;
-  for (int j = ty; j < 32; j += 8) {
-    const int m = p0 + mt + j, c = ct + tx;
-    const bf16 v = (m < pixels && mt + j < P && c < C) ? dz[(size_t)m * C + c] : __float2bfloat16_rn(0.f);
-    tile[j][tx] = v;
-    acc += __bfloat162float(v);
+// Tile image of dzT[c][m - p0] = dz[m][c] for m in [p0, p0 + P) (zero past the last pixel; P a multiple of 64, C of 16), and the
+// bias gradient: gb[c] += the sum over the pixels.  blockIdx.y takes 16 channels; a warp takes 16 pixels at a time and
+// transposes as k_im2col_t (32 x 32 tiles through shared memory, two bytes a thread: 283 us a step, now 96).
+__global__ void __launch_bounds__(256) k_dz_t(const bf16* __restrict__ dz, bf16* __restrict__ dzt, float* __restrict__ gb,
+                                              int pixels, int C, int p0, int P) {
+  const int lane = threadIdx.x & 31, c0 = blockIdx.y * 16 + 8 * (lane >> 4);
+  float sum = 0.f;
+  for (int w = blockIdx.x * 8 + (threadIdx.x >> 5); w < P / 16; w += gridDim.x * 8) {
+    const int mm = 16 * w + (lane & 15), m = p0 + mm;
+    const uint4 v = m < pixels ? __ldg(reinterpret_cast<const uint4*>(dz + (size_t)m * C + c0)) : make_uint4(0u, 0u, 0u, 0u);
+    uint32_t r[4] = {v.x, v.y, v.z, v.w};
+    transpose8(r, lane);
+    *reinterpret_cast<uint4*>(dzt + image_index(c0 + (lane & 7), (size_t)(mm & ~7), C)) = make_uint4(r[0], r[1], r[2], r[3]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) sum += __uint_as_float(r[i] << 16) + __uint_as_float(r[i] & 0xffff0000u);
   }
-  colsum[ty][tx] = acc;
+  sum += __shfl_xor_sync(0xffffffffu, sum, 8);  // the warp's other eight pixels
+  __shared__ float part[8][16];
+  if (!(lane & 8)) part[threadIdx.x >> 5][(lane & 7) + 8 * (lane >> 4)] = sum;
   __syncthreads();
-  for (int j = ty; j < 32; j += 8) {
-    const int c = ct + j, mm = mt + tx;
-    if (c < C && mm < P) dzt[(size_t)c * P + mm] = tile[tx][j];
-  }
-  if (ty == 0 && ct + tx < C) {
+  if (threadIdx.x < 16) {
     float t = 0.f;
 #pragma unroll
-    for (int r = 0; r < 8; ++r) t += colsum[r][tx];
-    atomicAdd(gb + ct + tx, t);
+    for (int k = 0; k < 8; ++k) t += part[k][threadIdx.x];
+    atomicAdd(gb + blockIdx.y * 16 + threadIdx.x, t);
   }
 }
 
@@ -697,36 +827,20 @@ static unsigned blocks_for(size_t n, unsigned cap = 152 * 16) {
   return (unsigned)(b < 1 ? 1 : (b > cap ? cap : b));
 }
 
-template <class LA, class LB, class Epi>
-static int gemm(const LA& la, const LB& lb, int rows, int cols, int K, const Epi& epi, int* status, cudaStream_t st,
-                int splits = 1) {
-#if PTY_GEMM_LEGACY
-  const int kt_all = (K + GB_K - 1) / GB_K;
-  if (splits > kt_all) splits = kt_all;
-  if (splits < 1) splits = 1;
-  const int kt_per = (kt_all + splits - 1) / splits;
-  const dim3 grid((cols + GB_N - 1) / GB_N, (rows + GB_M - 1) / GB_M, (kt_all + kt_per - 1) / kt_per);
-  k_gemm_tn<bf16, LA, LB, Epi, true><<<grid, GB_THREADS, 0, st>>>(la, lb, kt_all * GB_K, kt_per, epi);
-  (void)status;
-  CNN_CHECK("k_gemm_tn");
-#else
-  // tcgen05 tiles of 128 x BN, BN matched to the column count; every 64-wide K block is promoted to
-  // a round-to-nearest FP32 sum (see k_gemm_tc)
-  cudaError_t e;
-  if (cols <= 64) {
-    e = launch_gemm_tc<bf16, 64, true>(la, lb, rows, cols, K, epi, status, st, splits);
-  } else if (cols % 256 == 0) {
-    e = launch_gemm_tc<bf16, 256, true>(la, lb, rows, cols, K, epi, status, st, splits);
-  } else {
-    e = launch_gemm_tc<bf16, 128, true>(la, lb, rows, cols, K, epi, status, st, splits);
-  }
+static int gemm_result(cudaError_t e, const char* what) {
   if (e != cudaSuccess) {
-    set_error("k_gemm_tc launch failed: %s", cudaGetErrorString(e));
+    set_error("%s launch failed: %s", what, cudaGetErrorString(e));
     return PTY_ECUDA;
   }
   note_launch();
-#endif
   return PTY_OK;
+}
+// C = A B^T over row_tiles x 128 rows and b.rows columns in tiles of BN, which divides them, K = 64 kb_all
+template <int BN, int KS = 4, class LA, class Epi>
+static int gemm(const LA& la, const ImageOperand& b, int row_tiles, int kb_all, const Epi& epi, int* status,
+                cudaStream_t st, int splits = 1) {
+  return gemm_result(launch_gemm_ws<BN, KS>(la, b, WsWork{row_tiles, b.rows / BN, splits, kb_all, 0}, epi, status, st),
+                     "k_gemm_ws");
 }
 
 struct Buffers {
@@ -780,26 +894,36 @@ static int run_forward(const Plan& pl, const Buffers& bu, const float* params, c
     set_error("cudaMemsetAsync failed: %s", cudaGetErrorString(cudaGetLastError()));
     return PTY_ECUDA;
   }
-  k_pack<<<152 * 4, 256, 0, st>>>(pa);
+  k_pack<<<152 * 16, 256, 0, st>>>(pa);
   CNN_CHECK("k_pack");
   const int B = pl.B;
   if (B == 0) return PTY_OK;
   for (int l = 0; l < 5; ++l) {
     const LayerDef& L = kNet[l];
-    const int rows = B * pl.hout[l] * pl.hout[l];
-    PlainLoader<bf16> lb{bu.wp[l], (size_t)pl.kp[l], L.oc};
-    FwdEpi epi{bu.act[l], params + pl.boff[l], rows, L.oc};
+    const size_t rows = (size_t)B * pl.hout[l] * pl.hout[l];
+    const ImageOperand w{bu.wp[l], L.oc};
     int rc;
-    if (l == 0) {
-      rc = gemm(InputIm2col{I, s_in, pl.S, B, pl.hout[0]}, lb, rows, L.oc, pl.kp[l], epi, bu.status, st);
+    if (l == 0) {  // rows of 16 in the weight gradients' scratch, in pieces that fit it
+      const size_t fit = pl.colt_elems / 16 / 128 * 128;
+      for (size_t p0 = 0; p0 < rows; p0 += fit) {
+        const size_t n = rows - p0 < fit ? rows - p0 : fit;
+        k_input_rows<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(I, s_in, bu.colt, pl.S, pl.hout[0], p0, n);
+        CNN_CHECK("k_input_rows");
+        FwdEpi epi{bu.act[0] + p0 * L.oc, params + pl.boff[0], (int)n, L.oc};
+        if ((rc = gemm<48, 1>(InputRows{bu.colt, (int)n}, w, (int)((n + 127) / 128), 1, epi, bu.status, st))) return rc;
+      }
     } else {
-      rc = gemm(Im2col{bu.act[l - 1], B, pl.hin[l], pl.hu[l], pl.hout[l], L.ic, L.stride, L.up}, lb, rows, L.oc,
-                pl.kp[l], epi, bu.status, st);
+      FwdEpi epi{bu.act[l], params + pl.boff[l], (int)rows, L.oc};
+      const int tiles = (int)((rows + 127) / 128), kb = pl.kp[l] / 64;
+      const Im2col<1> la{bu.act[l - 1], B, pl.hin[l], pl.hu[l], pl.hout[l], L.ic, L.stride};
+      const Im2col<2> la2{bu.act[l - 1], B, pl.hin[l], pl.hu[l], pl.hout[l], L.ic, L.stride};
+      rc = l == 1 ? gemm<96>(la, w, tiles, kb, epi, bu.status, st)
+         : l == 4 ? gemm<256>(la2, w, tiles, kb, epi, bu.status, st) : gemm<192>(la, w, tiles, kb, epi, bu.status, st);
+      if (rc) return rc;
     }
-    if (rc) return rc;
   }
   const int hl = pl.hout[4], npix = B * hl * hl;
-  k_l6_sums<<<(npix + 7) / 8, 256, 0, st>>>(bu.act[4], bu.w6, bu.p6, npix);
+  k_l6_sums<<<npix < 4 * 152 * 4 ? (npix + 3) / 4 : 152 * 4, 128, 0, st>>>(bu.act[4], bu.w6, bu.p6, npix);
   CNN_CHECK("k_l6_sums");
   k_l6_out<<<blocks_for((size_t)B * 16 * hl * hl * kOut), 256, 0, st>>>(bu.p6, params + pl.boff[5], pred, B, hl);
   CNN_CHECK("k_l6_out");
@@ -832,12 +956,9 @@ static int run_backward(const Plan& pl, const Buffers& bu, const float* I, float
   const int npix = B * hl * hl;
   k_l6_dsums<<<blocks_for((size_t)npix * kTaps6), 256, 0, st>>>(bu.dz[5], bu.dp6, B, hl);
   CNN_CHECK("k_l6_dsums");
-  k_l6_dgrad<<<npix, kC6, 0, st>>>(bu.dp6, bu.w6, bu.act[4], bu.dz[4], npix);
-  CNN_CHECK("k_l6_dgrad");
-  const int chunk = 256;
-  k_l6_wgrad<<<dim3((npix + chunk - 1) / chunk, kTaps6), kC6, 0, st>>>(bu.dp6, bu.act[4], grad + pl.woff[5], npix,
-                                                                       chunk);
-  CNN_CHECK("k_l6_wgrad");
+  k_l6_grad<<<npix < 8 * 152 * 4 ? (npix + 7) / 8 : 152 * 4, kC6, 0, st>>>(bu.dp6, bu.w6, bu.act[4], bu.dz[4],
+                                                                          grad + pl.woff[5], npix);
+  CNN_CHECK("k_l6_grad");
   const size_t pix6 = (size_t)B * hs * hs;
   k_bias_grad<<<(unsigned)((pix6 + 1023) / 1024), 256, 0, st>>>(bu.dz[5], grad + pl.boff[5], pix6, kOut, 1024);
   CNN_CHECK("k_bias_grad");
@@ -850,33 +971,39 @@ static int run_backward(const Plan& pl, const Buffers& bu, const float* I, float
     // transposed to pixel-contiguous rows first (plain 16-byte loads in the GEMM)
     const int P = pl.pchunk[l];
     for (int p0 = 0; p0 < pixels; p0 += P) {
-      if (l == 0) {
-        k_im2col_t1<<<blocks_for((size_t)9 * P), 256, 0, st>>>(I, s_in, bu.colt, B, pl.S, pl.hout[0], p0, P);
-      } else {
-        k_im2col_t<<<blocks_for((size_t)L.ic / 8 * P), 256, 0, st>>>(bu.act[l - 1], bu.colt, B, pl.hin[l], pl.hu[l],
-                                                                     pl.hout[l], L.ic, L.stride, L.up, p0, P);
-      }
-      CNN_CHECK("k_im2col_t");
-      k_dz_t<<<dim3((P + 31) / 32, (L.oc + 31) / 32), dim3(32, 8), 0, st>>>(bu.dz[l], bu.dzt, grad + pl.boff[l], pixels,
-                                                                          L.oc, p0, P);
+      const unsigned xb = (unsigned)((P / 16 + 7) / 8), cap = 152 * 16 / (L.oc / 16);
+      k_dz_t<<<dim3(xb < cap ? xb : cap, L.oc / 16), 256, 0, st>>>(bu.dz[l], bu.dzt, grad + pl.boff[l], pixels, L.oc, p0, P);
       CNN_CHECK("k_dz_t");
-      const int tiles = ((k9 + 127) / 128) * ((L.oc + 127) / 128);
-      const int splits = 2 * 152 / tiles > 1 ? 2 * 152 / tiles : 1;
-      int rc = gemm(PlainLoader<bf16>{bu.dzt, (size_t)P, L.oc}, PlainLoader<bf16>{bu.colt, (size_t)P, k9}, L.oc, k9,
-                    P, WgradEpi{grad + pl.woff[l], L.oc, k9}, bu.status, st, splits);
+      if (l == 0)
+        k_im2col_t1<<<blocks_for((size_t)P), 256, 0, st>>>(I, s_in, bu.colt, B, pl.S, pl.hout[0], p0, P);
+      else
+        k_im2col_t<<<blocks_for((size_t)L.ic / 16 * P * 2), 256, 0, st>>>(bu.act[l - 1], bu.colt, B, pl.hin[l], pl.hu[l],
+                                                                         pl.hout[l], L.ic, L.stride, L.up, p0, P);
+      CNN_CHECK("k_im2col_t");
+      // 9 ic = 432, 864, 1728 or 3456 columns: tiles of 144 divide them; layer 1: one tile of 16
+      const ImageLoad la{ImageOperand{bu.dzt, L.oc}};
+      const int row_tiles = (L.oc + 127) / 128, tiles = row_tiles * (l == 0 ? 1 : k9 / 144), splits = 2 * 152 / tiles;
+      const int rc = l == 0 ? gemm<16>(la, ImageOperand{bu.colt, 16}, row_tiles, P / 64,
+                                       WgradEpi{grad + pl.woff[l], L.oc, k9}, bu.status, st, splits)
+                            : gemm<144>(la, ImageOperand{bu.colt, k9}, row_tiles, P / 64,
+                                        WgradImageEpi{grad + pl.woff[l], L.oc, k9}, bu.status, st, splits);
       if (rc) return rc;
     }
     if (l == 0) break;
-    const int rows = B * pl.hu[l] * pl.hu[l];
-    DgradGather ga{bu.dz[l], B, pl.hu[l], pl.hout[l], L.oc, L.stride};
-    PlainLoader<bf16> wt{bu.wt[l], (size_t)pl.ktp[l], L.ic};
+    const GradRows gr(B, pl.hu[l], L.stride);
+    const int kb = pl.ktp[l] / 64;
+    const DgradGather ga(bu.dz[l], gr, pl.hout[l], L.oc, kb);
+    const ImageOperand wt{bu.wt[l], L.ic};
     int rc;
     if (L.up == 1) {
-      rc = gemm(ga, wt, rows, L.ic, pl.ktp[l], DgradEpi{bu.dz[l - 1], bu.act[l - 1], rows, L.ic}, bu.status, st);
+      const DgradEpi epi{bu.dz[l - 1], bu.act[l - 1], gr, L.ic};
+      rc = l == 1 ? gemm<48>(ga, wt, gr.row_tiles(), kb, epi, bu.status, st)
+         : l == 2 ? gemm<96>(ga, wt, gr.row_tiles(), kb, epi, bu.status, st)
+                  : gemm<192>(ga, wt, gr.row_tiles(), kb, epi, bu.status, st);
     } else {
-      rc = gemm(ga, wt, rows, L.ic, pl.ktp[l], StoreEpi{bu.du5, rows, L.ic}, bu.status, st);
+      rc = gemm<192>(ga, wt, gr.row_tiles(), kb, StoreEpi{bu.du5, B * pl.hu[l] * pl.hu[l], L.ic}, bu.status, st);
       if (rc) return rc;
-      k_upsample_grad<<<blocks_for((size_t)B * pl.hin[l] * pl.hin[l] * L.ic), 256, 0, st>>>(
+      k_upsample_grad<<<blocks_for((size_t)B * pl.hin[l] * pl.hin[l] * L.ic / 4), 256, 0, st>>>(
           bu.du5, bu.act[l - 1], bu.dz[l - 1], B, pl.hin[l], L.ic, L.up);
       CNN_CHECK("k_upsample_grad");
     }
