@@ -437,33 +437,52 @@ struct WgradEpi {  // the same for layer 1 (nine columns)
 // ---------------------------------------------------------------------------------------------
 // Layer 6 on the CUDA cores
 // ---------------------------------------------------------------------------------------------
-// P[p][j] = sum_c w6[j][c] a5[p][c]: one warp per low-resolution pixel, 8 channels per lane; a warp keeps its lanes'
-// weights in registers over all its pixels (loaded through shared memory by every 8 pixels: 97 us on 65536).
+// P[p][j] = sum_c w6[j][c] a5[p][c]: one warp per low-resolution pixel, 8 channels per lane, weights in registers over
+// all of a warp's pixels.  The eighteen sums over lanes are halved along with the lanes (20 shuffles; the same
+// additions as eighteen butterflies, whose 90 shuffles one after the other took 102 us on 65536 pixels; 33 here).
+template <int NV>
+__device__ __forceinline__ void halve(float* t, int o, bool upper) {
+  constexpr int H = (NV + 1) / 2;
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    const float hi = i + H < NV ? t[i + H] : 0.f;
+    t[i] = (upper ? hi : t[i]) + __shfl_xor_sync(0xffffffffu, upper ? t[i] : hi, o);
+  }
+}
 __global__ void __launch_bounds__(128) k_l6_sums(const bf16* __restrict__ a5, const float* __restrict__ w6,
                                                  float* __restrict__ P, int npix) {
-  const int lane = threadIdx.x & 31;
+  static_assert(kTaps6 == 18, "the halving below");
+  const int lane = threadIdx.x & 31, step = gridDim.x * 4;
   float w[kTaps6][8];
 #pragma unroll
   for (int j = 0; j < kTaps6; ++j)
 #pragma unroll
     for (int e = 0; e < 8; ++e) w[j][e] = __ldg(w6 + j * kC6 + lane * 8 + e);
-  for (int p = blockIdx.x * 4 + (threadIdx.x >> 5); p < npix; p += gridDim.x * 4) {
-    Pack8 v;
-    v.u = __ldg(reinterpret_cast<const uint4*>(a5 + (size_t)p * kC6 + lane * 8));
-    float x[8];
+  // 18 -> 9 -> 5 -> 3 -> 2 -> 1 values: the one that this lane ends with, if it is one
+  const int i4 = lane & 1, i3 = i4 + (lane & 2), i2 = i3 + (lane & 4 ? 3 : 0), i1 = i2 + (lane & 8 ? 5 : 0);
+  const int mine = i1 + (lane & 16 ? 9 : 0);
+  const bool valid = i3 < 3 && i2 < 5 && i1 < 9;
+  int p = blockIdx.x * 4 + (threadIdx.x >> 5);
+  Pack8 v, nv;
+  if (p < npix) nv.u = __ldg(reinterpret_cast<const uint4*>(a5 + (size_t)p * kC6 + lane * 8));
+  for (; p < npix; p += step) {
+    v = nv;
+    if (p + step < npix) nv.u = __ldg(reinterpret_cast<const uint4*>(a5 + (size_t)(p + step) * kC6 + lane * 8));
+    float t[kTaps6];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) x[e] = __bfloat162float(v.h[e]);
-    float mine = 0.f;
+    for (int j = 0; j < kTaps6; ++j) t[j] = 0.f;
 #pragma unroll
-    for (int j = 0; j < kTaps6; ++j) {
-      float t = 0.f;
+    for (int e = 0; e < 8; ++e) {
+      const float x = __bfloat162float(v.h[e]);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) t = fmaf(w[j][e], x[e], t);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      if (lane == j) mine = t;
+      for (int j = 0; j < kTaps6; ++j) t[j] = fmaf(w[j][e], x, t[j]);
     }
-    if (lane < kTaps6) P[(size_t)p * kTaps6 + lane] = mine;
+    halve<18>(t, 16, lane & 16);
+    halve<9>(t, 8, lane & 8);
+    halve<5>(t, 4, lane & 4);
+    halve<3>(t, 2, lane & 2);
+    halve<2>(t, 1, lane & 1);
+    if (valid) P[(size_t)p * kTaps6 + mine] = t[0];
   }
 }
 
@@ -506,12 +525,17 @@ __global__ void __launch_bounds__(256) k_loss(const float* __restrict__ pred, co
   }
   if (threadIdx.x == 0) lpart[blockIdx.x] = red[0];
 }
-__global__ void k_loss_final(const double* __restrict__ lpart, int nb, size_t n, double* loss) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double t = 0.0;
-    for (int i = 0; i < nb; ++i) t += lpart[i];
-    *loss = t / (double)n;
+__global__ void __launch_bounds__(256) k_loss_final(const double* __restrict__ lpart, int nb, size_t n, double* loss) {
+  __shared__ double red[256];
+  double t = 0.0;
+  for (int i = threadIdx.x; i < nb; i += 256) t += lpart[i];
+  red[threadIdx.x] = t;
+  __syncthreads();
+  for (int h = 128; h > 0; h >>= 1) {
+    if ((int)threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
+    __syncthreads();
   }
+  if (threadIdx.x == 0) *loss = red[0] / (double)n;
 }
 
 // dP[p][tap][o] = sum of dz6 over the output pixels that read low-resolution pixel p through tap:
@@ -950,7 +974,7 @@ static int run_backward(const Plan& pl, const Buffers& bu, const float* I, float
   const unsigned lb = blocks_for(nout, 1024);
   k_loss<<<lb, 256, 0, st>>>(pred, Y, bu.dz[5], bu.lpart, nout);
   CNN_CHECK("k_loss");
-  k_loss_final<<<1, 32, 0, st>>>(bu.lpart, (int)lb, nout, loss);
+  k_loss_final<<<1, 256, 0, st>>>(bu.lpart, (int)lb, nout, loss);
   CNN_CHECK("k_loss_final");
   // layer 6
   const int npix = B * hl * hl;

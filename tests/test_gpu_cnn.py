@@ -204,6 +204,38 @@ def test_each_layer_matches_oracle_on_the_gpu_inputs(S, B):
             _assert_bf16_close(dz[l - 1], C.bf16(dx * (acts[l - 1] > 0)), ("dz", l - 1))
 
 
+@pytest.mark.parametrize("S,B", [(48, 7), (80, 3), (112, 2)])
+def test_each_layer_at_tile_edges(S, B):
+    """Row counts that end inside the GEMMs' 128-row tiles, in every parity class of the input gradients."""
+    test_each_layer_matches_oracle_on_the_gpu_inputs(S, B)
+
+
+def test_smallest_network_matches_oracle():
+    test_forward_matches_oracle(16, 1)
+
+
+def test_wait_that_runs_out_returns_etimeout_and_the_next_call_is_clean():
+    from paper_2505_07814_gb300 import _lib
+    net, _ = _net(64, 3)
+    I, Y = (torch.tensor(x, device="cuda") for x in _data(64, 3))
+    want, pred = torch.empty((3, 32, 32, 2), device="cuda"), torch.empty((3, 32, 32, 2), device="cuda")
+
+    def status():
+        return _lib.pty_status(net.ws.data_ptr(), torch.cuda.current_stream().cuda_stream)
+
+    net.loss_grad(I, Y, pred=want)
+    assert status() == 0
+    try:
+        _lib.pty_set_wait_limit(0)
+        net.loss_grad(I, Y, pred=pred)
+        st = status()
+    finally:
+        _lib.pty_set_wait_limit(-1)
+    assert st >= 0 and st & _lib.PTY_ETIMEOUT, st
+    net.loss_grad(I, Y, pred=pred)
+    assert status() == 0 and torch.equal(pred, want)
+
+
 def test_learned_start_reaches_target_nmse_sooner_than_flat_start():
     """Trained on 16384 forward-model pairs from four random volumes (not the test object), the
     network's stitched start is closer to the truth than the flat start and the reconstruction
