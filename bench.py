@@ -767,7 +767,7 @@ def roofline_of(wl, args, stage_ms, ncalls, sms, clocks, fma_tflops):
     except (OSError, ValueError):
         pass
     return {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-            "traffic": None, "kernel": "k_gemm_tc (every DFT GEMM of the pass)", "avg_pass_ms": avg_ms,
+            "traffic": None, "kernel": "k_dft_gemm (every DFT GEMM of the pass)", "avg_pass_ms": avg_ms,
             "peak_source": "MEASURED_PEAKS.json bf16_tflops (burst; fp16 taken equal)"}
 
 

@@ -720,32 +720,9 @@ __global__ void k_stitch_finish(int Nz, int H, int W, const float* __restrict__ 
   }
 }
 
-
 // ---------------------------------------------------------------------------------------------
 // Weight-gradient operands with pixel-contiguous rows
 // ---------------------------------------------------------------------------------------------
-// Transpose of 8 x 8 16-bit values over eight consecutive lanes: lane p's r[i] holds values 2 i, 2 i + 1 of row p; afterwards
-// of column p.
-__device__ __forceinline__ void transpose8(uint32_t (&r)[4], int lane) {
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const uint32_t o = __shfl_xor_sync(0xffffffffu, r[i], 1);
-    r[i] = (lane & 1) ? __byte_perm(o, r[i], 0x7632) : __byte_perm(r[i], o, 0x5410);
-  }
-#pragma unroll
-  for (int i = 0; i < 4; i += 2) {
-    const uint32_t o = __shfl_xor_sync(0xffffffffu, (lane & 2) ? r[i] : r[i + 1], 2);
-    if (lane & 2) r[i] = o;
-    else r[i + 1] = o;
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const uint32_t o = __shfl_xor_sync(0xffffffffu, (lane & 4) ? r[i] : r[i + 2], 4);
-    if (lane & 4) r[i] = o;
-    else r[i + 2] = o;
-  }
-}
-
 // Tile image of colT[k][m - p0] = im2col[m][k] for k = (tap, ic) < 9 IC and output pixels m in [p0, p0 + P); zero past the
 // last pixel (layers 2..5, ic a multiple of 16).  A warp takes 16 pixels by two groups of 8 channels: per tap each
 // lane loads its pixel's 16 bytes, eight lanes transpose 8 pixels x 8 channels, and every store is one core

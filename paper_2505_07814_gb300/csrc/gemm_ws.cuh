@@ -1,7 +1,6 @@
 // gemm_ws.cuh -- C = A * B^T on the 5th-generation tensor cores with a role for every warp, for the learned
-// initialiser's layers.  Same arithmetic as k_gemm_tc (gemm_tc.cuh): K in blocks of 64, each summed by the tensor
-// cores into a fresh TMEM region and added to FP32 registers with round-to-nearest adds, in K order, so the
-// results are the same bits.
+// initialiser's layers.  K in blocks of 64, each summed by the tensor cores into a fresh TMEM region and added to
+// FP32 registers with round-to-nearest adds, in K order.
 //
 // One CTA of eleven warps per SM, which takes the 128 x BN tiles blockIdx.x, + gridDim.x, ...:
 //   warps 0-7   promote: read a finished block's TMEM region, add it to their registers, run the epilogue;
@@ -11,8 +10,8 @@
 //               issues the bulk copies of operands that are kept as tile images (B always; A when it is one);
 //   warp 10     one thread issues the MMAs.
 // Stages pass between them on mbarriers, so the loads of later blocks and tiles, the MMAs and the promotion
-// overlap; k_gemm_tc's eight warps did all three in turn, one block ahead, with two barriers a block: the
-// 65536 x 256 x 3456 layer took 5500 clocks a block where its MMAs need 512 (507 us; 238 here).
+// overlap; where eight warps do all three in turn, one block ahead, with two barriers a block, the
+// 65536 x 256 x 3456 layer takes 5500 clocks a block where its MMAs need 512 (507 us; 238 here).
 //
 // Tile images.  An operand of R rows (a multiple of 8) is stored by K block: block kb holds, for every 8 rows, the
 // eight 8 x 8 core matrices along K (128 bytes each), which is the tensor core's canonical K-major layout without
@@ -97,6 +96,28 @@ __device__ __forceinline__ bool ws_wait(uint32_t bar, uint32_t parity, long limi
     if ((i & 63) == 63 && *abort) return false;
   }
   return false;
+}
+
+// Transpose of 8 x 8 16-bit values over eight consecutive lanes: lane p's r[i] holds values 2 i, 2 i + 1 of row p; afterwards
+// of column p.
+__device__ __forceinline__ void transpose8(uint32_t (&r)[4], int lane) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t o = __shfl_xor_sync(0xffffffffu, r[i], 1);
+    r[i] = (lane & 1) ? __byte_perm(o, r[i], 0x7632) : __byte_perm(r[i], o, 0x5410);
+  }
+#pragma unroll
+  for (int i = 0; i < 4; i += 2) {
+    const uint32_t o = __shfl_xor_sync(0xffffffffu, (lane & 2) ? r[i] : r[i + 1], 2);
+    if (lane & 2) r[i] = o;
+    else r[i + 1] = o;
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const uint32_t o = __shfl_xor_sync(0xffffffffu, (lane & 4) ? r[i] : r[i + 2], 4);
+    if (lane & 4) r[i] = o;
+    else r[i + 2] = o;
+  }
 }
 
 // Work of one launch: row tiles x column tiles x splits of K, columns fastest (CTAs side by side share A's rows).

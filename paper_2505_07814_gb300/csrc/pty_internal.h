@@ -40,7 +40,7 @@ struct Workspace {
   double* pacpart; // [B][N / 32]     sums of I_meas^p_pacbed
   double* sppart;  // [152*8]         partial sums of c |phase|^p_sparse (sparsity term)
   int* cover;      // [H][W+1]        patch coverage count c of the batch (sparsity term)
-  void* pieces0;   // [B][M][N][pieces][2N] 16-bit split operands of the tensor-core GEMMs
+  void* pieces0;   // [pieces][2N / 64] tile images of [waves * N][64]: 16-bit split operand of the DFT GEMMs
   void* pieces1;   // (the same, for the second GEMM of a 2D transform)
 };
 

@@ -88,6 +88,20 @@ def test_split_single_slice_global_tilt(fft):
     _assert(_errors(case, list(range(case.Ntot)), fft), fft)
 
 
+@pytest.mark.parametrize("fft", FORMATS)
+@pytest.mark.parametrize("N,M,scan,B", [(64, 1, (1, 1), 1), (64, 3, (9, 12), 105), (128, 1, (1, 1), 1), (128, 1, (9, 9), 79)])
+def test_split_patterns_at_tile_edges(fft, N, M, scan, B):
+    """One tile, a last tile half full (an odd number of 64-row waves), and more tiles than CTAs: the patterns agree
+    with the FP32 transforms' to the intensity bar."""
+    case = make_case(N=N, M=M, Nz=2, scan=scan, seed=16)
+    out = {}
+    for f in (fft, "fp32"):
+        pt, params, _ = _gpu(case, f)
+        out[f] = _np(pt.forward(params, list(range(B))))
+        assert pt.status() == 0
+    assert rel_l2(out[fft], out["fp32"]) <= TOL_I
+
+
 def test_split_ignores_ckpt_stride_and_matches_fp32_path():
     """ckpt_stride > 1 does not change the split modes; the two precisions agree with the FP32 FFT
     path to well inside their own tolerance."""
