@@ -222,9 +222,10 @@ struct InputRows {
     int tap, off;
   };
   __device__ __forceinline__ const bf16* any() const { return x16; }
+  __device__ __forceinline__ int tile_class(int) const { return 0; }
   __device__ __forceinline__ int kb_next(int, int kb) const { return kb; }
   __device__ __forceinline__ GatherRow row(int m) const { return GatherRow{x16 + (size_t)m * 16, m < rows ? 1u : 0u, 0u}; }
-  __device__ __forceinline__ K kpos(int k) const { return K{0, k}; }
+  __device__ __forceinline__ K kpos(int k, int) const { return K{0, k}; }
   __device__ __forceinline__ int offset(const GatherRow&, const K& k) const { return k.off; }
 };
 
@@ -240,6 +241,7 @@ struct Im2col {
     int tap, y[UP], x[UP];  // elements, by the parity of the pixel; x holds the channel too
   };
   __device__ __forceinline__ const bf16* any() const { return a; }
+  __device__ __forceinline__ int tile_class(int) const { return 0; }
   __device__ __forceinline__ int kb_next(int, int kb) const { return kb; }
   __device__ __forceinline__ GatherRow row(int m) const {
     if (m >= B * hout * hout) return GatherRow{a, 0u, 0u};
@@ -253,7 +255,7 @@ struct Im2col {
     const long long pix = (long long)(b * hin + (y0 >> (UP - 1))) * hin + (x0 >> (UP - 1));
     return GatherRow{a + pix * ic, mask, 0u};
   }
-  __device__ __forceinline__ K kpos(int k) const {
+  __device__ __forceinline__ K kpos(int k, int) const {
     K r;
     r.tap = k / ic;
     const int ky = r.tap / 3, kx = r.tap - 3 * ky;
@@ -311,12 +313,12 @@ struct DgradGather {
     }
   }
   struct K {
-    int tap, y, x;  // (ky, kx) for stride 2; y the whole offset for stride 1
+    int tap, offset;
   };
+  __device__ __forceinline__ int tile_class(int tile) const { return g.tile_class(tile); }
   __device__ __forceinline__ const bf16* any() const { return dz; }
-  __device__ __forceinline__ int kb_next(int tile, int kb) const {
+  __device__ __forceinline__ int kb_next(int c, int kb) const {
     if (g.stride == 1) return kb;
-    const int c = g.tile_class(tile);
     const unsigned long long left = (c == 0 ? blocks[0] : c == 1 ? blocks[1] : c == 2 ? blocks[2] : blocks[3]) >> kb;  // kb <= 54
     return left ? kb + __ffsll((long long)left) - 1 : 64;
   }
@@ -337,19 +339,15 @@ struct DgradGather {
           mask |= 1u << t;
       }
     }
-    mask |= (unsigned)cls << 16;
     return GatherRow{dz + ((size_t)(b * hout + y) * hout + x) * oc, mask, 0u};
   }
-  __device__ __forceinline__ K kpos(int k) const {
+  // a tap's offset is the same for every row of a class
+  __device__ __forceinline__ K kpos(int k, int cls) const {
     const int tap = k / oc, ky = tap / 3, kx = tap - 3 * ky, o = k - tap * oc;
-    if (g.stride == 1) return K{tap, ((1 - ky) * hout + 1 - kx) * oc + o, 0};
-    return K{tap, ky, (o << 2) | kx};
+    if (g.stride == 1) return K{tap, ((1 - ky) * hout + 1 - kx) * oc + o};
+    return K{tap, ((((cls >> 1) + 1 - ky) >> 1) * hout + (((cls & 1) + 1 - kx) >> 1)) * oc + o};
   }
-  __device__ __forceinline__ int offset(const GatherRow& r, const K& k) const {
-    if (g.stride == 1) return k.y;
-    const int py = r.m >> 17 & 1, px = r.m >> 16 & 1;
-    return (((py + 1 - k.y) >> 1) * hout + ((px + 1 - (k.x & 3)) >> 1)) * oc + (k.x >> 2);
-  }
+  __device__ __forceinline__ int offset(const GatherRow&, const K& k) const { return k.offset; }
 };
 struct ImageLoad {
   static constexpr bool kGather = false;

@@ -129,6 +129,7 @@ struct DftShape {
   static constexpr int B_BLOCK = 192 * 128, B_BYTES = KB * PC * B_BLOCK, STAGE = 128 * 128;
   static constexpr int STAGES = (229376 - B_BYTES) / STAGE < 8 ? (229376 - B_BYTES) / STAGE : 8;
   static constexpr size_t SMEM = (size_t)B_BYTES + STAGES * STAGE + 1024 + 256;
+  static_assert(8 * (2 * STAGES + 9) + 8 <= 256, "barriers, TMEM slot, abort flag");
   static constexpr size_t TABLE = (size_t)PARTS * B_BYTES / 2;  // elements of one matrix
 };
 

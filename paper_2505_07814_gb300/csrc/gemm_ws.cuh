@@ -2,16 +2,16 @@
 // initialiser's layers.  K in blocks of 64, each summed by the tensor cores into a fresh TMEM region and added to
 // FP32 registers with round-to-nearest adds, in K order.
 //
-// One CTA of eleven warps per SM, which takes the 128 x BN tiles blockIdx.x, + gridDim.x, ...:
+// One CTA per SM, which takes the 128 x BN tiles blockIdx.x, + gridDim.x, ...:
 //   warps 0-7   promote: read a finished block's TMEM region, add it to their registers, run the epilogue;
-//   warps 8, 9  gather the A tile with cp.async (im2col rows: 8 rows x 64 bytes a warp instruction), two blocks
+//   2 or 4 warps gather the A tile with cp.async (im2col rows: 8 rows x 64 bytes a warp instruction), two blocks
 //               behind their own loads when they announce a stage; a row is a pointer and a mask of its
 //               valid taps, decoded once per tile, so a chunk costs a bit test and an add.  One thread also
 //               issues the bulk copies of operands that are kept as tile images (B always; A when it is one);
-//   warp 10     one thread issues the MMAs.
+//   last warp   one thread issues the MMAs.
 // Stages pass between them on mbarriers, so the loads of later blocks and tiles, the MMAs and the promotion
 // overlap; where eight warps do all three in turn, one block ahead, with two barriers a block, the
-// 65536 x 256 x 3456 layer takes 5500 clocks a block where its MMAs need 512 (507 us; 238 here).
+// 65536 x 256 x 3456 layer takes 5500 clocks a block where its MMAs need 512 (507 us; 230 here).
 //
 // Tile images.  An operand of R rows (a multiple of 8) is stored by K block: block kb holds, for every 8 rows, the
 // eight 8 x 8 core matrices along K (128 bytes each), which is the tensor core's canonical K-major layout without
@@ -25,7 +25,7 @@
 
 namespace pty {
 
-constexpr int WS_THREADS = 352, WS_PROMOTE = 256, WS_GATHER = 64;
+constexpr int WS_PROMOTE = 256;
 constexpr int kWsBlock = 64;  // K per block and tile image
 
 // Element (row, k) of a tile-image operand of `rows` rows, in elements.
@@ -45,10 +45,11 @@ struct WsShape {
   static constexpr int REGION = BN <= 64 ? 64 : BN <= 128 ? 128 : 256;  // TMEM columns of a region
   static constexpr int A_BYTES = 128 * 128, B_BYTES = BN * 128, STAGE = A_BYTES + B_BYTES;
   static constexpr int STAGES = 196608 / STAGE < 8 ? 196608 / STAGE : 8;
-  static constexpr int ROWS_BYTES = 2 * 128 * 16;  // the gathering warps' row tables
+  static constexpr int ROWS_BYTES = 2 * 128 * 16;  // the gathering warps' row tables (two per row)
   static constexpr size_t SMEM = (size_t)STAGES * STAGE + 1024 + 256 + ROWS_BYTES;
+  static_assert(8 * (3 * STAGES + 4) + 8 <= 256, "barriers, TMEM slot, abort flag");
   static constexpr int HALF = BN / 2;  // columns of a promoting warp
-  static constexpr int CH = HALF % 32 == 0 ? 32 : HALF % 24 == 0 ? 24 : 8;  // columns read from TMEM at a time
+  static constexpr int CH = HALF == 96 ? 16 : HALF % 32 == 0 ? 32 : HALF % 24 == 0 ? 24 : 8;  // columns read from TMEM at a time
   static_assert(BN % 16 == 0 && HALF % CH == 0 && BN <= 256 && STAGES >= 4, "tile");
 };
 
@@ -120,6 +121,19 @@ __device__ __forceinline__ void transpose8(uint32_t (&r)[4], int lane) {
   }
 }
 
+// Warps that gather A (or, where A is an image, issue its copies).  A warp spends ~60 clocks a cp.async on addresses
+// and masks one after the other; with two warps the MMAs of the narrow layers waited 2100 clocks a block for A
+// (input gradients of 48 and 96 columns: 497 and 210 us with two warps, 264 and 122 with four).  At 256 columns the
+// promoting warps' 128 sums leave no registers for two more warps (238 us with two, 480 with four and spills).
+template <class LoadA, int BN>
+__host__ __device__ constexpr int ws_gather_warps() {
+  return !LoadA::kGather ? 1 : BN <= 192 ? 4 : 2;
+}
+template <class LoadA, int BN>
+__host__ __device__ constexpr int ws_threads() {
+  return WS_PROMOTE + 32 * ws_gather_warps<LoadA, BN>() + 32;
+}
+
 // Work of one launch: row tiles x column tiles x splits of K, columns fastest (CTAs side by side share A's rows).
 struct WsWork {
   int row_tiles, col_tiles, splits, kb_all, kb_per;
@@ -132,15 +146,15 @@ struct GatherRow {
   unsigned m;
   unsigned pad;
 };
-// LoadA: gathered operands define kGather = true, GatherRow row(int m), K kpos(int k) with a member tap, int offset(row, K)
-// in elements, and int kb_next(int tile, int kb): the first block >= kb with a nonzero element in the row tile (skipped
-// blocks would add exact zeros).  Image operands: kGather = false, member `op`.
+// LoadA: gathered operands define kGather = true, GatherRow row(int m), int tile_class(int tile), K kpos(int k, int cls)
+// with a member tap, int offset(row, K) in elements, and int kb_next(int cls, int kb): the first block >= kb with a
+// nonzero element in row tiles of the class (skipped blocks would add exact zeros).  Image operands: kGather = false, member `op`.
 // Epi: Row prep(int m) and epi(Row, col, v) with eight consecutive columns.
 template <class LoadA, class Epi, int BN, int KS>
-__global__ void __launch_bounds__(WS_THREADS, 1)
+__global__ void __launch_bounds__(ws_threads<LoadA, BN>(), 1)
     k_gemm_ws(LoadA la, ImageOperand b, WsWork wk, Epi epi, int* status, long spin) {
   using S = WsShape<BN, KS>;
-  constexpr int ST = S::STAGES;
+  constexpr int ST = S::STAGES, GW = ws_gather_warps<LoadA, BN>();
   extern __shared__ __align__(1024) unsigned char ws_raw[];
   unsigned char* base = (unsigned char*)(((uintptr_t)ws_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* bars = reinterpret_cast<uint64_t*>(base + ST * S::STAGE);
@@ -158,7 +172,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
   if (tid == 0) {
     auto init = [](uint32_t bar, int n) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(n)); };
     for (int i = 0; i < ST; ++i) {
-      init(fullA + 8 * i, WS_GATHER);
+      init(fullA + 8 * i, 32 * GW);
       init(fullB + 8 * i, 1);
       init(empty + 8 * i, 1);
     }
@@ -176,7 +190,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
 
   const int items = wk.row_tiles * wk.col_tiles * wk.splits;
   struct Item {
-    int tile, n0, kb0, kb1;
+    int tile, n0, kb0, kb1, cls;
   };
   auto item = [&](int w) {
     Item it;
@@ -185,10 +199,11 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
     const int z = w / wk.col_tiles / wk.row_tiles;
     it.kb0 = z * wk.kb_per;
     it.kb1 = min(it.kb0 + wk.kb_per, wk.kb_all);
+    if constexpr (LoadA::kGather) it.cls = la.tile_class(it.tile);
     return it;
   };
   auto next = [&](const Item& it, int kb) {  // first block >= kb of the item with work, or kb1
-    if constexpr (LoadA::kGather) return min(la.kb_next(it.tile, kb), it.kb1);
+    if constexpr (LoadA::kGather) return min(la.kb_next(it.cls, kb), it.kb1);
     else return kb;
   };
   auto fail = [&]() {
@@ -227,7 +242,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
 #pragma unroll
       for (int j = 0; j < S::HALF; j += 8) epi(row, it.n0 + col0 + j, acc + j);
     }
-  } else if (warp < 10) {
+  } else if (warp < 8 + GW) {
     // ---- gather A; bulk copies ----
     const int t = tid - WS_PROMOTE;
     const bool copies = t == 0;
@@ -236,12 +251,13 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
     for (int w = blockIdx.x; w < items && ok; w += gridDim.x) {
       const Item it = item(w);
       if constexpr (LoadA::kGather) {
-        const int kg = (lane >> 3) + 4 * (warp & 1);
-        constexpr int ROWS = 16;
-        GatherRow* table = reinterpret_cast<GatherRow*>(base + ST * S::STAGE + 256) + 128 * (warp & 1);
+        // warp pairs take 256 / GW rows each, the two warps of a pair four of the eight 16-byte chunks of K
+        const int kg = (lane >> 3) + 4 * (warp & 1), row0 = ((warp - 8) >> 1) * (256 / GW);
+        constexpr int ROWS = 32 / GW;
+        GatherRow* table = reinterpret_cast<GatherRow*>(base + ST * S::STAGE + 256) + (256 / GW) * (warp - 8);
         __syncwarp();
 #pragma unroll
-        for (int j = 0; j < 4; ++j) table[lane + 32 * j] = la.row(it.tile * 128 + lane + 32 * j);
+        for (int j = 0; j < ROWS / 4; ++j) table[lane + 32 * j] = la.row(it.tile * 128 + row0 + lane + 32 * j);
         __syncwarp();
         GatherRow row[ROWS];
 #pragma unroll
@@ -259,8 +275,8 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
             ws_bulk(tc_smem_u32(st + S::A_BYTES), b.p + (size_t)kb * b.rows * 64 + (size_t)it.n0 * 64, S::B_BYTES, fullB + 8 * s);
           }
           if (KS == 4 || kg < 2 * KS) {
-            const typename LoadA::K k = la.kpos(kb * kWsBlock + 8 * kg);
-            const uint32_t d = tc_smem_u32(st) + (lane & 7) * 16 + kg * 128;
+            const typename LoadA::K k = la.kpos(kb * kWsBlock + 8 * kg, it.cls);
+            const uint32_t d = tc_smem_u32(st) + row0 * 128 + (lane & 7) * 16 + kg * 128;
 #pragma unroll
             for (int j = 0; j < ROWS; ++j) {
               const bool in = (row[j].m >> k.tap) & 1;
@@ -359,7 +375,7 @@ cudaError_t launch_gemm_ws(const LA& la, const ImageOperand& b, WsWork wk, const
   wk.kb_per = (wk.kb_all + wk.splits - 1) / wk.splits;
   wk.splits = (wk.kb_all + wk.kb_per - 1) / wk.kb_per;
   const long long items = (long long)wk.row_tiles * wk.col_tiles * wk.splits;
-  kern<<<(unsigned)(items < 152 ? items : 152), WS_THREADS, S::SMEM, st>>>(la, b, wk, epi, status, stage_wait_limit());
+  kern<<<(unsigned)(items < 152 ? items : 152), ws_threads<LA, BN>(), S::SMEM, st>>>(la, b, wk, epi, status, stage_wait_limit());
   return cudaGetLastError();
 }
 
