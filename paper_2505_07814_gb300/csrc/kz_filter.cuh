@@ -20,7 +20,7 @@
 // convolution of the column with a real kernel h(d) = sum_k W_a(k) cos(2 pi k d / Nz), h(d) = h(Nz - d):
 // 2 FMAs per pair of slices where the two DFTs take 8.
 //
-// Measured (GB300, one call; the start is one radix-2 stage per barrier, direct DFTs for other lengths, a DFT
+// Measured (GB300, one call; before: one radix-2 stage per barrier, direct DFTs for other lengths, a DFT
 // pair over depth): 20 x 1024 x 1024 1954 -> 751 us, 6 x 614 x 614 5226 -> 256 us.  The five passes
 // move 88 bytes per voxel: 2.5 TB/s on the large volume, bound by the latency of each tile's load,
 // barrier-separated passes and store with two CTAs on an SM; the ragged lines are bound by their arithmetic.
