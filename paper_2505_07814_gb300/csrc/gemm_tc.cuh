@@ -56,6 +56,14 @@ __device__ __forceinline__ bool tc_wait(uint32_t bar, uint32_t parity, long limi
 // TC_SPIN); pty_set_wait_limit changes it for tests that make a wait run out.
 long stage_wait_limit();
 
+// Completes this warp's tensor-memory loads into r.  The loads are asynchronous and only their own asm statements name r,
+// so without the statements after the wait a use of r could be placed before it.
+template <int N>
+__device__ __forceinline__ void tc_ld_wait(uint32_t (&r)[N]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int j = 0; j < N; ++j) asm volatile("" : "+r"(r[j]));
+}
 __device__ __forceinline__ void tc_ld32(uint32_t taddr, float* v) {
   uint32_t r[32];
   asm volatile(
@@ -66,7 +74,7 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, float* v) {
         "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
         "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  tc_ld_wait(r);
 #pragma unroll
   for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
 }

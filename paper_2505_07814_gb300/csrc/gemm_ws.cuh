@@ -69,12 +69,9 @@ __device__ __forceinline__ void tc_ld_add(uint32_t taddr, float* acc) {
     uint32_t r[CH];
 #pragma unroll
     for (int j = 0; j < CH; j += 8) tc_ld8_nowait(taddr + j, r + j);
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    tc_ld_wait(r);
 #pragma unroll
-    for (int j = 0; j < CH; ++j) {
-      asm volatile("" : "+r"(r[j]));  // not before the wait
-      acc[j] += __uint_as_float(r[j]);
-    }
+    for (int j = 0; j < CH; ++j) acc[j] += __uint_as_float(r[j]);
   }
 }
 __device__ __forceinline__ void ws_arrive(uint32_t bar) {
