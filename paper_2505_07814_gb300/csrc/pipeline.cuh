@@ -205,12 +205,16 @@ __device__ __forceinline__ Pair pair_warp_sum(Pair x) {
     x = pair_add(x, Pair{__shfl_down_sync(0xffffffffu, x.hi, o), __shfl_down_sync(0xffffffffu, x.lo, o)});
   return x;
 }
-// a sum that overflowed stays infinite (its lo is not a number)
-__device__ __forceinline__ double pair_total(Pair x) {
-  return isfinite(x.hi) ? (double)x.hi + (double)x.lo : (double)x.hi;
+// (a sum with a finite hi: a hi beyond a float's range is infinite or not a number, and its sum has to be formed in FP64)
+__device__ __forceinline__ double pair_total(Pair x) { return (double)x.hi + (double)x.lo; }
+__device__ __forceinline__ double warp_sum(double x) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+  return x;
 }
 // Sums of NV values over the CTA's T threads, each in the thread of its number (threads < NV), in pairs of floats
-// and a fixed order (an FP64 shuffle sum costs 64 clocks of a scheduler per step and value).  red: NV * T / 32 pairs.
+// and a fixed order (an FP64 shuffle sum costs 64 clocks of a scheduler per step and value), in FP64 where one of
+// them leaves a float's range.  red: NV * T / 32 pairs, aligned for doubles.
 template <int T, int NV>
 __device__ __forceinline__ double block_sum_pairs(const float (&v)[NV], Pair* red) {
   constexpr int W = T / 32;
@@ -230,7 +234,20 @@ __device__ __forceinline__ double block_sum_pairs(const float (&v)[NV], Pair* re
       if (lane == q) r = Pair{hi, lo};
     }
   }
-  return threadIdx.x < NV ? pair_total(r) : 0.0;
+  if (__syncthreads_or(!isfinite(r.hi))) {
+    double* wide = reinterpret_cast<double*>(red);
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+      const double x = warp_sum((double)v[q]);
+      if (lane == 0) wide[q * W + w] = x;
+    }
+    __syncthreads();
+    double x = 0.0;
+    if (threadIdx.x < NV)
+      for (int i = 0; i < W; ++i) x += wide[threadIdx.x * W + i];
+    return x;
+  }
+  return pair_total(r);
 }
 // exp(i pi (hi + lo)): hi reduced modulo 2 exactly, lo as a first-order rotation while its second order, (pi lo)^2 / 2, is
 // below 2e-8.  That is so up to phases of about a thousand half turns; a lo of more than 2^-14 is first
@@ -1103,7 +1120,7 @@ __global__ void __launch_bounds__(4 * N, 256 / N) k_loss(LossArgs a) {
   constexpr int T = 4 * N, NN = N * N, S = loss_parts<N>(), RS = 33;
   constexpr int PX = 8, E4 = PX / 4;  // pixels and float4s a thread
   __shared__ float L[N * RS];
-  __shared__ Pair red[3 * (T / 32)];
+  __shared__ __align__(8) Pair red[3 * (T / 32)];
   __shared__ double fin[16];
   __shared__ int last;
   const int b = blockIdx.x / S, s = blockIdx.x % S, tid = threadIdx.x;
@@ -1773,8 +1790,13 @@ __global__ void __launch_bounds__(T, Launch<N>::MINB_A) k_adjoint(AdjArgs a) {
     Pair x{0.f, 0.f};
     for (int i = lane; i < T; i += 32) x = pair_add(x, Pair{part[q * T + i], 0.f});
     x = pair_warp_sum(x);
+    double sum = pair_total(x);
+    if (!isfinite(__shfl_sync(0xffffffffu, x.hi, 0))) {  // beyond a float's range: in FP64
+      sum = 0.0;
+      for (int i = lane; i < T; i += 32) sum += (double)part[q * T + i];
+      sum = warp_sum(sum);
+    }
     if (lane == 0) {
-      const double sum = pair_total(x);
       if constexpr (F::C == 1) {
         a.spart[(size_t)bm * 5 + q] += sum;
       } else {  // the CTAs of a cluster each hold part of the wave
