@@ -312,7 +312,9 @@ int pty_loss_grad_noalloc(const pty_geom* geom, int B, const int32_t* idx, const
  *   of calls recorded, or -1 on a CUDA error.  Stages: 0 prepare_object, 1 probe_spectrum, 2 forward,
  *   3 loss, 4 loss_finalize, 5 adjoint, 6 object_grad, 7 probe_grad, 8 scalar_grad.  Work that shares
  *   a launch is counted in the first of its stages (0 holds 1 and 6 holds 7 and 8 for objects up to
- *   8 Mi voxels at N <= 128; 3 always holds 4). */
+ *   8 Mi voxels at N <= 128; 3 always holds 4).  Kernels without a stage count in the next stage that
+ *   ran: the PACBED term's in 5; the sparsity term's in 7 or 8, whichever runs next, and in 8 when
+ *   the probe's and the scalars' gradients were made before it or not at all. */
 #define PTY_PROF_STAGES 9
 long long pty_launch_count(void);
 int pty_profile_enable(int on);

@@ -2474,6 +2474,8 @@ struct Pass {
       PTY_LAUNCH_CHECK("k_object_grad", 6);
     }
     if (pb.mode == MODE_GRAD && pb.w_sp > 0.f && ws.sppart && pb.B > 0) {
+      // no later kernel of the call to be counted with: a stage mark of its own
+      const int last = rest && (want_probe || scalars) ? -1 : 8;
       // coverage count of the batch's patches, then one pass over every slice of every object mode
       if (cudaMemsetAsync(ws.cover, 0, sizeof(int) * (size_t)pb.H * (pb.W + 1), st) != cudaSuccess)
         return memset_failed();
@@ -2486,14 +2488,14 @@ struct Pass {
       PTY_LAUNCH_CHECK("k_sparse_sum", -1);
       k_sparse_finalize<<<1, 256, 0, st>>>(ws.sppart, kSparseBlocks, patch_pixels, pb.p_sp, pb.w_sp, pb.loss_out,
                                            ws.scal, ws.status);
-      PTY_LAUNCH_CHECK("k_sparse_finalize", -1);
+      PTY_LAUNCH_CHECK("k_sparse_finalize", last);
       if ((gm & PTY_GRAD_PHASE) && pb.g_phase) {
         if (!want_obj && !pb.accumulate &&
             cudaMemsetAsync(pb.g_phase, 0, sizeof(float) * nobj(), st) != cudaSuccess)
           return memset_failed();
         k_sparse_grad<<<object_blocks(), 256, 0, st>>>(pb.phase, ws.cover, pb.H, pb.W, nobj(), pb.p_sp, pb.w_sp,
                                                        ws.scal, pb.g_phase);
-        PTY_LAUNCH_CHECK("k_sparse_grad", -1);
+        PTY_LAUNCH_CHECK("k_sparse_grad", last);
       }
     }
     if (rest && want_probe) {
