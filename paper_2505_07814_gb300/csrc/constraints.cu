@@ -109,6 +109,19 @@ __global__ void k_constrain(float* __restrict__ x0, float* __restrict__ x1, int 
   }
 }
 
+// The dynamic shared memory that launches of `kern` may ask for.  The limit belongs to the function and not to a launch, and
+// host threads with other sizes share it: every call that needs more than the default sets the same number, the
+// largest that any call needs.
+template <class Kern>
+static int allow_smem(Kern kern, size_t bytes, size_t largest, const char* what) {
+  if (bytes > 48 * 1024 &&
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)largest) != cudaSuccess) {
+    set_error("cudaFuncSetAttribute(%s) failed: %s", what, cudaGetErrorString(cudaGetLastError()));
+    return PTY_ECUDA;
+  }
+  return PTY_OK;
+}
+
 template <int V>
 static int launch_constrain(float* amp, float* phase, int Nz, size_t plane, float sigma, float rz_relax,
                             float pos_relax, cudaStream_t st) {
@@ -120,11 +133,7 @@ static int launch_constrain(float* amp, float* phase, int Nz, size_t plane, floa
     T = (int)((kConstrainSmem - fixed) / ((size_t)Nz * V * sizeof(float)));
     T = T >= 128 ? 128 : T / 32 * 32;
     smem = fixed + (size_t)Nz * T * V * sizeof(float);
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(k_constrain<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-      set_error("cudaFuncSetAttribute(k_constrain) failed: %s", cudaGetErrorString(cudaGetLastError()));
-      return PTY_ECUDA;
-    }
+    if (int rc = allow_smem(k_constrain<V>, smem, kConstrainSmem, "k_constrain")) return rc;
   }
   const int R0 = (int)ceilf(4.0f * sigma);
   const int R = blur ? (R0 < Nz - 1 ? R0 : Nz - 1) : 0;
@@ -469,16 +478,6 @@ static int check_constraints(const pty_geom* geom, const pty_constraints* c) {
   return PTY_OK;
 }
 
-template <class Kern>
-static int big_smem(Kern kern, size_t smem, const char* what) {
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-    set_error("cudaFuncSetAttribute(%s) failed: %s", what, cudaGetErrorString(cudaGetLastError()));
-    return PTY_ECUDA;
-  }
-  return PTY_OK;
-}
-
 // One pass of line transforms.  C lines per tile, a power of two up to 8 while two CTAs fit an SM, at least
 // one; as many CTAs as fit the chip at once take the tiles in turn.
 template <int MODE, int KIND>
@@ -489,8 +488,7 @@ static int run_lines_of(KzArgs a, cudaStream_t st) {
   while (a.C > 1 && tables + kz_lines_bytes(a.line, a.C) > kKzSmem / 2) a.C /= 2;
   const size_t smem = tables + kz_lines_bytes(a.line, a.C);
   a.tiles = X ? (long long)a.Nz * ((a.H + a.C - 1) / a.C) : (long long)((a.W + 7) / 8) * a.Nz * (8 / a.C);
-  int rc = big_smem(k_kz_lines<MODE, KIND>, smem, "k_kz_lines");
-  if (rc) return rc;
+  if (int rc = allow_smem(k_kz_lines<MODE, KIND>, smem, kKzSmem, "k_kz_lines")) return rc;
   long long per_sm = (long long)(kKzSmem / (smem + 1024));
   per_sm = per_sm < 1 ? 1 : per_sm > 4 ? 4 : per_sm;
   const long long grid = a.tiles < 152 * per_sm ? a.tiles : 152 * per_sm;
@@ -521,7 +519,7 @@ static int run_kz_filter(const pty_geom* g, float* amp, float* phase, const floa
   a.line = ly;
   if ((rc = run_lines<KZ_Y_FWD>(a, st))) return rc;
   const size_t smem = kz_depth_bytes(g->Nz);
-  if ((rc = big_smem(k_kz_depth, smem, "k_kz_depth"))) return rc;
+  if ((rc = allow_smem(k_kz_depth, smem, kz_depth_bytes(kMaxBlurSlices), "k_kz_depth"))) return rc;
   const int columns = g->H * (g->W < 8 ? g->W : 8);  // of a block
   k_kz_depth<<<dim3((columns + kDepthThreads - 1) / kDepthThreads, (g->W + 7) / 8), kDepthThreads, smem, st>>>(
       z, g->Nz, g->H, g->W, g->dx, dz, c->kz_beta, c->kz_alpha, lx, ly);
@@ -539,15 +537,15 @@ static int run_orthogonalize(const pty_geom* g, float* probe, const ConstrainLay
   double* lam = reinterpret_cast<double*>(ws + L.lam);
   float2* P = reinterpret_cast<float2*>(probe);
   int rc;
-  const size_t gram_smem = sizeof(double2) * ((size_t)kGramTile * M + 256);
-  if ((rc = big_smem(k_gram, gram_smem, "k_gram"))) return rc;
-  k_gram<<<chunks, 256, gram_smem, st>>>(P, M, NN, partial);
+  auto gram_smem = [](int m) { return sizeof(double2) * ((size_t)kGramTile * m + 256); };
+  auto apply_smem = [](int m) { return sizeof(double2) * ((size_t)m * m + (size_t)m * 128); };
+  if ((rc = allow_smem(k_gram, gram_smem(M), gram_smem(kMaxOrthoModes), "k_gram"))) return rc;
+  k_gram<<<chunks, 256, gram_smem(M), st>>>(P, M, NN, partial);
   if ((rc = launched("k_gram"))) return rc;
   k_ortho_eig<<<1, 256, 0, st>>>(partial, M, chunks, U, lam);
   if ((rc = launched("k_ortho_eig"))) return rc;
-  const size_t smem = sizeof(double2) * ((size_t)M * M + (size_t)M * 128);
-  if ((rc = big_smem(k_ortho_apply, smem, "k_ortho_apply"))) return rc;
-  k_ortho_apply<<<(NN + 127) / 128, 128, smem, st>>>(P, M, NN, U);
+  if ((rc = allow_smem(k_ortho_apply, apply_smem(M), apply_smem(kMaxOrthoModes), "k_ortho_apply"))) return rc;
+  k_ortho_apply<<<(NN + 127) / 128, 128, apply_smem(M), st>>>(P, M, NN, U);
   return launched("k_ortho_apply");
 }
 

@@ -170,3 +170,36 @@ def test_constrain_rejects_unsupported_sizes():
     for kw in (dict(kz_beta=-1.0, kz_relax=1.0), dict(kz_beta=1.0, kz_relax=1.5), dict(kz_alpha=float("inf"))):
         with pytest.raises(_lib.PtyError):
             constrain(pt, params, **kw)
+
+
+def test_two_threads_with_different_sizes():
+    """Two host threads, each with its own problem, stream and workspace: neither's launches may depend on the
+    shared-memory sizes that the other's need.  64 object modes make a call some 500 launches long, so that the
+    threads' launches meet."""
+    import threading
+
+    from paper_2505_07814_gb300.ptycho import Geometry, Params, Ptycho, constrain
+    errors = []
+
+    def work(M, Nz, W):
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            z = lambda *s: torch.zeros(s, device="cuda")  # noqa: E731
+            geom = Geometry(N=64, M=M, Nz=Nz, H=64, W=W, Ntot=1, dx=0.1, lam=0.025, grads=(), obj_modes=64)
+            params = Params(z(64, Nz, 64, W) + 1, z(64, Nz, 64, W), torch.randn((M, 64, 64), dtype=torch.complex64, device="cuda"),
+                            z(1, 2), z(1, 2), z(1) + 2)
+            pt = Ptycho(geom, 1)
+            for i in range(30):
+                try:
+                    constrain(pt, params, rz_sigma=0.5, kz_beta=0.8, kz_alpha=0.01, kz_relax=0.9, orthogonalize_probe=True)
+                except Exception as e:  # noqa: BLE001
+                    errors.append((M, i, str(e)))
+                stream.synchronize()
+
+    threads = [threading.Thread(target=work, args=a) for a in ((32, 60, 80), (24, 40, 66))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors, (len(errors), errors[:3])
