@@ -174,7 +174,9 @@ __global__ void __launch_bounds__(256) k_gram(const float2* __restrict__ probe, 
   extern __shared__ __align__(16) double2 g_px[];  // [kGramTile][M], then [256] partial sums
   double2* red = g_px + (size_t)kGramTile * M;
   const int tid = threadIdx.x, np = M * (M + 1) / 2, c0 = blockIdx.x * kGramChunk;
-  const int groups = np < 256 ? 256 / np : 1;  // np <= 528: up to three pairs a thread
+  // np <= 528: up to three pairs a thread.  M = 2 and 3 take 16 shares a pair instead of 85 and 42, whose addition
+  // one after the other was most of the pass (N = 64: 9.6 and 8.0 us, now 6.5 and 6.7)
+  const int groups = np < 8 ? 16 : np < 256 ? 256 / np : 1;
   const int grp = np < 256 ? tid / np : 0;
   double re[3] = {0.0, 0.0, 0.0}, im[3] = {0.0, 0.0, 0.0};
   int pm[3], pn[3], cnt = 0;

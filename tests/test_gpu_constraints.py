@@ -203,3 +203,9 @@ def test_two_threads_with_different_sizes():
         t.join()
     torch.cuda.synchronize()
     assert not errors, (len(errors), errors[:3])
+
+
+@pytest.mark.parametrize("M,N", [(2, 64), (2, 256), (3, 64)])
+def test_orthogonalize_two_and_three_modes(M, N):
+    """The Gram pass with 16 shares a mode pair."""
+    test_orthogonalize_probe_matches_oracle(M, N)
