@@ -2174,10 +2174,12 @@ struct Pass {
   unsigned object_blocks() const {
     return (unsigned)((nobj() + 255) / 256 < 152 * 16 ? (nobj() + 255) / 256 : 152 * 16);
   }
-  // Whether the object's passes share a launch with the probe's transforms.  The launch then has the
-  // transforms' shared memory, so an SM holds few of its CTAs; that costs nothing while the object's
-  // arrays fit L2 (8 Mi voxels: 64 MB of T), and saves a launch and the wait between two small kernels
-  // (64 x 64, one mode, 128 x 128 object: 3.3 + 5.6 us as two kernels, 3.8 as one).
+  // Whether the object's passes share a launch with the probe's transforms.  That saves two launches at each end of
+  // a call and the waits between small kernels; but the launch has the transforms' shared memory, so an SM holds few
+  // of its CTAs, and with a large object the passes over it run below their bandwidth.  One gradient call, 4
+  // positions, shared / separate: N = 64, one mode, object of 1, 8, 16, 64 Mi voxels 79 / 99, 219 / 240, 384 / 398,
+  // 1385 / 1393 us; N = 128, two modes, 1, 8, 16, 32, 64 Mi 107 / 130, 402 / 412, 700 / 705, 1297 / 1295, 2498 / 2473.
+  // 8 Mi lies below the crossing at either size.
   bool together() const { return C == 1 && nobj() <= ((size_t)8 << 20); }
   unsigned shared_blocks() const {  // CTAs of T threads for the object in such a launch, four elements a thread
     const size_t b = (nobj() + 4 * T - 1) / (4 * T), per = N == 64 ? 4 : 1;
