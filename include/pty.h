@@ -281,8 +281,9 @@ int pty_supported_sizes(void);
  * a real-time loop that cannot afford the device-wide synchronisation of cudaMalloc / cudaFree.
  * There is no counterpart in the paper; the computation is exactly pty_loss_grad's.
  *  - Scratch is a fixed array of PTY_NOALLOC_SCRATCH_BYTES (32 MiB) inside this library's device
- *    code.  Every GPU that loads the library holds it until the process exits.  A batch whose
- *    pty_workspace_size() exceeds it is rejected with PTY_EWORKSPACE before anything is launched.
+ *    code, with 256 KiB on top for the wave tables' constants and the loss kernel's partial sums.  Every
+ *    GPU that loads the library holds it until the process exits.  A batch whose workspace without
+ *    those two pieces exceeds 32 MiB is rejected with PTY_EWORKSPACE before anything is launched.
  *    The workspace holds the transmission and its gradient (16 bytes per object voxel) besides the
  *    per-wave buffers, so the object alone must stay under 2 Mi voxels (for example 8 x 512 x 512
  *    does not fit, 1 x 1024 x 1024 fits with a few 64 x 64 waves).
