@@ -11,7 +11,7 @@
 //   last warp   one thread issues the MMAs.
 // Stages pass between them on mbarriers, so the loads of later blocks and tiles, the MMAs and the promotion
 // overlap; where eight warps do all three in turn, one block ahead, with two barriers a block, the
-// 65536 x 256 x 3456 layer takes 5500 clocks a block where its MMAs need 512 (507 us; 230 here).
+// 65536 x 256 x 3456 layer takes 5500 clocks a block where its MMAs need 512 (507 us; 232 here).
 //
 // Tile images.  An operand of R rows (a multiple of 8) is stored by K block: block kb holds, for every 8 rows, the
 // eight 8 x 8 core matrices along K (128 bytes each), which is the tensor core's canonical K-major layout without
@@ -121,7 +121,7 @@ __device__ __forceinline__ void transpose8(uint32_t (&r)[4], int lane) {
 // Warps that gather A (or, where A is an image, issue its copies).  A warp spends ~60 clocks a cp.async on addresses
 // and masks one after the other; with two warps the MMAs of the narrow layers waited 2100 clocks a block for A
 // (input gradients of 48 and 96 columns: 497 and 210 us with two warps, 264 and 122 with four).  At 256 columns the
-// promoting warps' 128 sums leave no registers for two more warps (238 us with two, 480 with four and spills).
+// promoting warps' 128 sums leave no registers for two more warps (232 us with two, 480 with four and spills).
 template <class LoadA, int BN>
 __host__ __device__ constexpr int ws_gather_warps() {
   return !LoadA::kGather ? 1 : BN <= 192 ? 4 : 2;
