@@ -212,11 +212,11 @@ __device__ __forceinline__ double warp_sum(double x) {
   for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
   return x;
 }
-// Sums of NV values over the CTA's T threads, each in the thread of its number (threads < NV), in pairs of floats
-// and a fixed order (an FP64 shuffle sum costs 64 clocks of a scheduler per step and value), in FP64 where one of
-// them leaves a float's range.  red: NV * T / 32 pairs, aligned for doubles.
+// Sums of NV values over the CTA's T threads, each in the thread of its number (threads < NV; zero in the first warp's
+// others), in pairs of floats and a fixed order (an FP64 shuffle sum costs 64 clocks of a scheduler per step and
+// value).  red: NV * T / 32 pairs.
 template <int T, int NV>
-__device__ __forceinline__ double block_sum_pairs(const float (&v)[NV], Pair* red) {
+__device__ __forceinline__ Pair block_sum_pairs(const float (&v)[NV], Pair* red) {
   constexpr int W = T / 32;
   const int lane = threadIdx.x & 31, w = threadIdx.x / 32;
 #pragma unroll
@@ -234,28 +234,35 @@ __device__ __forceinline__ double block_sum_pairs(const float (&v)[NV], Pair* re
       if (lane == q) r = Pair{hi, lo};
     }
   }
-  if (__syncthreads_or(!isfinite(r.hi))) {
-    double* wide = reinterpret_cast<double*>(red);
+  return r;
+}
+// The same in FP64, for sums that leave a float's range.  red: NV * T / 32 doubles.
+template <int T, int NV>
+__device__ __forceinline__ double block_sum_wide(const float (&v)[NV], double* red) {
+  constexpr int W = T / 32;
 #pragma unroll
-    for (int q = 0; q < NV; ++q) {
-      const double x = warp_sum((double)v[q]);
-      if (lane == 0) wide[q * W + w] = x;
-    }
-    __syncthreads();
-    double x = 0.0;
-    if (threadIdx.x < NV)
-      for (int i = 0; i < W; ++i) x += wide[threadIdx.x * W + i];
-    return x;
+  for (int q = 0; q < NV; ++q) {
+    const double x = warp_sum((double)v[q]);
+    if ((threadIdx.x & 31) == 0) red[q * W + threadIdx.x / 32] = x;
   }
-  return pair_total(r);
+  __syncthreads();
+  double x = 0.0;
+  if (threadIdx.x < NV)
+    for (int i = 0; i < W; ++i) x += red[threadIdx.x * W + i];
+  return x;
 }
 // exp(i pi (hi + lo)): hi reduced modulo 2 exactly, lo as a first-order rotation while its second order, (pi lo)^2 / 2, is
 // below 2e-8.  That is so up to phases of about a thousand half turns; a lo of more than 2^-14 is first
 // added to the reduced hi without loss, and what their sum rounds off is the rotation (of 2^17 half turns lo reaches
 // 2^-7, an error of 3e-4 in the modulus without it).
+// FAR false: phases of a few half turns, whose lo is always small.
+template <bool FAR = true>
 __device__ __forceinline__ float2 expipi(Pair x) {
-  const float big = fabsf(x.lo) > 6.103515625e-5f ? x.lo : 0.f;
-  const Pair p = pair_add(Pair{x.hi - 2.0f * rintf(0.5f * x.hi), 0.f}, Pair{big, x.lo - big});
+  Pair p{x.hi - 2.0f * rintf(0.5f * x.hi), x.lo};
+  if constexpr (FAR) {
+    const float big = fabsf(x.lo) > 6.103515625e-5f ? x.lo : 0.f;
+    p = pair_add(Pair{p.hi, 0.f}, Pair{big, x.lo - big});
+  }
   float s, c;
   sincospif(p.hi, &s, &c);
   const float d = 3.14159265358979f * p.lo;
@@ -265,7 +272,7 @@ __device__ __forceinline__ float2 expipi(Pair x) {
 template <int N>
 __device__ __forceinline__ float2 ramp(float f, float q, float d) {
   const float p = __fmul_rn(q, d), w = f / (float)N;  // w: a power of two
-  return expipi(Pair{p * w, fmaf(q, d, -p) * w});
+  return expipi<false>(Pair{p * w, fmaf(q, d, -p) * w});
 }
 
 // Signed DFT frequency index of bin k.
@@ -1199,17 +1206,26 @@ __global__ void __launch_bounds__(4 * N, 256 / N) k_loss(LossArgs a) {
   for (int e = tid; e < 32 * N; e += T)
     a.u[(size_t)b * NN + (e / 32) * N + 32 * s + e % 32] = L[(e / 32) * RS + loss_col<N>(e / 32, e % 32)];
   const float v3[3] = {sd, st, sp};
-  const double sum = block_sum_pairs<T>(v3, red);
-  if (tid < 2) a.lpart[2 * blockIdx.x + tid] = sum;
-  if (PAC && tid == 2) a.pacpart[blockIdx.x] = sum;
-  if (tid < 32) {  // the warp that wrote the sums counts the CTA as done
+  auto finish = [&](double sum) {  // first warp: the CTA's sums, then the CTA counts as done
+    if (tid < 2) a.lpart[2 * blockIdx.x + tid] = sum;
+    if (PAC && tid == 2) a.pacpart[blockIdx.x] = sum;
     __syncwarp();
     if (tid == 0) {
       __threadfence();
       last = atomicAdd(a.status + 1, 1) == (int)gridDim.x - 1;
     }
+  };
+  const Pair r = block_sum_pairs<T>(v3, red);
+  if (tid < 32) {
+    if (__all_sync(0xffffffffu, isfinite(r.hi))) finish(pair_total(r));
+    else if (tid == 0) last = -1;
   }
   __syncthreads();
+  if (last < 0) {  // a sum beyond a float's range
+    const double sum = block_sum_wide<T>(v3, reinterpret_cast<double*>(red));
+    if (tid < 32) finish(sum);
+    __syncthreads();
+  }
   if (!last) return;
   __threadfence();  // every CTA's sums are visible
   if (tid < 256) loss_finalize(a, (int)gridDim.x, fin);
@@ -1791,7 +1807,7 @@ __global__ void __launch_bounds__(T, Launch<N>::MINB_A) k_adjoint(AdjArgs a) {
     for (int i = lane; i < T; i += 32) x = pair_add(x, Pair{part[q * T + i], 0.f});
     x = pair_warp_sum(x);
     double sum = pair_total(x);
-    if (!isfinite(__shfl_sync(0xffffffffu, x.hi, 0))) {  // beyond a float's range: in FP64
+    if (__builtin_expect(!isfinite(__shfl_sync(0xffffffffu, x.hi, 0)), 0)) {  // beyond a float's range: in FP64
       sum = 0.0;
       for (int i = lane; i < T; i += 32) sum += (double)part[q * T + i];
       sum = warp_sum(sum);
